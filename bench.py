@@ -66,8 +66,10 @@ CPU_SAMPLE = (96, 256, 256)
 # capture), scaled by 4 to the 256 tiles of a launch of the bench's field
 # (the traffic grows with the tiles).
 NCU_TRAFFIC = {
-    ("field", "tf_arms"): {"bytes": 4 * (54528000 + 772520960), "digest": "451b42818bf0103a"},
-    ("field", "tf_psf_rows"): {"bytes": 4 * (906436096 + 440025600), "digest": "cf4d832d91af6988"},
+    ("field", "tf_arms"): {"bytes": 4 * (34782464 + 461256192), "digest": "17cb36cee354e9a9"},
+    ("field", "tf_psf_rows"): {"bytes": 4 * (584111616 + 420239104), "digest": "e44e6a6ce754cda6"},
+    ("field", "tf_yz"): {"bytes": 4 * (368271616 + 308391168), "digest": "05e5c2753d8d7fa1"},
+    ("field", "yz_op"): {"bytes": 4 * (742178816 + 403828224), "digest": "05e5c2753d8d7fa1"},
 }
 
 
@@ -77,10 +79,10 @@ def kernel_digest(name: str) -> str:
     src = {"z_fused": ["wo_zops.cuh", "wo_zops_a.cu", "wo_zops_b.cu", "wo_zreg.cu", "wo_regfft.cuh"],
            "z_solve2d": ["wo_zops.cuh", "wo_zops_a.cu"], "rows_r2c": ["wo_rows.cu"], "rows_c2r": ["wo_rows.cu"],
            "xy_fwd": ["wo_xy.cu", "wo_rowsplit.cuh", "wo_regfft.cuh"], "xy_inv": ["wo_xy.cu", "wo_rowsplit.cuh", "wo_regfft.cuh"],
-           "y_fwd": ["wo_cols.cu"], "y_inv": ["wo_cols.cu"], "tf_ypass": ["wo_cols.cu"], "tf_arms": tf + ["wo_armsreg.cu", "wo_regfft.cuh"],
+           "y_fwd": ["wo_cols.cu"], "y_inv": ["wo_cols.cu"], "tf_ypass": ["wo_cols.cu"], "tf_arms": tf + ["wo_tfeven.cu", "wo_armsreg.cu", "wo_regfft.cuh"],
            # the register-resident row kernel (rows of 32..512 points; wo_tf.cu holds only the
            # shared-memory fallback for other lengths)
-           "tf_psf_rows": ["wo_psf.cu", "wo_regfft.cuh", "wo_tf.cuh"],
+           "tf_psf_rows": ["wo_tfeven.cu", "wo_psf.cu", "wo_regfft.cuh", "wo_tf.cuh"],
            "tf_zpass": tf + ["wo_zops.cuh"],
            "tf_pupil_record": tf, "tune_cols": ["wo_tune.cu"],
            "tf_yz": ["wo_plane.cu", "wo_bulk.cuh", "wo_regfft.cuh", "wo_zops.cuh"],

@@ -133,7 +133,7 @@ static Layout layout_of(int n, int Z, int Y, int X, const Sys& s) {
   size_t off = L.head;
   L.optics = off; off += align256((size_t)n * sizeof(wo_optics));
   L.zern = off; if (s.aberr) off += align256((size_t)n * WO_MAX_ZERNIKE * sizeof(double));
-  L.counts = off; off += align256((size_t)n * 4 * sizeof(int));
+  L.counts = off; off += align256((size_t)n * kCounts * sizeof(int));
   L.rec = off; off += align256((size_t)n * Y * X * sizeof(float4));
   L.rec2 = off; if (s.want_grad || s.aberr) off += align256((size_t)n * Y * X * sizeof(float4));
   const int rb = (Y + record_rows(Y, n) - 1) / record_rows(Y, n);
@@ -433,7 +433,7 @@ static wo_status build_tf_impl(const wo_optics* optics, bool on_host, int n_tile
   if (s.aberr)
     WO_TRY(cudaMemcpyAsync((void*)a.zern, h_zern, (size_t)n_tiles * n_zern * sizeof(double), cudaMemcpyHostToDevice,
                            cs));
-  WO_TRY(cudaMemsetAsync(a.counts, 0, (size_t)n_tiles * 4 * sizeof(int), cs));
+  WO_TRY(cudaMemsetAsync(a.counts, 0, (size_t)n_tiles * kCounts * sizeof(int), cs));
   WO_TRY(cudaMemsetAsync(a.stats, 0, (size_t)n_tiles * 8 * sizeof(float), cs));
   WO_TRY(tf_pupil_record(a, cs));
   WO_TRY(tf_arms(a, cs));

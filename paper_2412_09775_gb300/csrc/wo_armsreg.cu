@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(ArmGeom<P>::NT) k_arms_reg(TfArgs a) {
   const int t = blockIdx.z, j = blockIdx.y, x0 = blockIdx.x * CPC;
   const int w = min(CPC, X - x0);
   // strips whose columns all lie outside the detection band: every arm is zero
-  const int kxmax = a.counts[4 * t + 2];
+  const int kxmax = a.counts[kCounts * t + kCntKx];
   bool active = false;
   for (int b = 0; b < w; ++b) active |= abs(fft_index(x0 + b, X)) <= kxmax;
   if (!active) return;  // uniform across the CTA

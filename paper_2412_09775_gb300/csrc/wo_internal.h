@@ -157,9 +157,10 @@ cudaError_t z_fuse(int Z, const float2* in, float2* out, const float2* tf, const
                    int Xh, cudaStream_t s);
 
 // Transfer-function build.
+constexpr int kCounts = 8;  // ints per tile of TfArgs::counts (named in wo_tf.cuh)
 struct TfArgs {
   const wo_optics* optics;  // device copy, [n_tiles]
-  int* counts;              // [n_tiles][4]: #(S and P) (binary source), #P, x band limit, -
+  int* counts;              // [n_tiles][kCounts]: pupil counts and bands (wo_tf.cuh)
   float4* rec;              // [n_tiles][Y][X] pupil record
   float2* arms;             // [n_tiles][n_arms][Z][Y][X]
   float2* tf;               // [n_tiles][n_kinds][Z][Y][Xh]
@@ -187,10 +188,16 @@ struct TfArgs {
 cudaError_t tf_pupil_record(const TfArgs& a, cudaStream_t s);
 int record_rows(int Y, int n_tiles);  // rows per pupil-record block
 cudaError_t tf_arms(const TfArgs& a, cudaStream_t s);
-// Arm pass with register-resident y transforms (wo_armsreg.cu): banks without derivatives, Y <= 192.
+// Arm pass with register-resident y transforms (wo_armsreg.cu): banks without derivatives, Y <= 192, where
+// tf_even_supported() is false (an aberrated pupil, other row lengths).
 bool arms_reg_supported(int Y, const TfArgs& a);
 cudaError_t tf_arms_reg(const TfArgs& a, cudaStream_t s);
 cudaError_t tf_psf_rows(const TfArgs& a, cudaStream_t s);
+// The arm and PSF-row passes of banks whose detection pupil is even in k_x
+// and k_y (wo_tfeven.cu).
+bool tf_even_supported(const TfArgs& a);
+cudaError_t tf_arms_even(const TfArgs& a, cudaStream_t s);
+cudaError_t tf_psf_rows_even(const TfArgs& a, cudaStream_t s);
 // The TF build's z pass for one-kind banks with register-resident z
 // transforms (wo_zreg.cu).
 bool tf_zpass_reg_supported(const TfArgs& a);

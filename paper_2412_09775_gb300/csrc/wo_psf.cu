@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4)
     }
   }
 #endif
-  const int kxm = a.counts[4 * t + 2];
+  const int kxm = a.counts[kCounts * t + kCntKx];
   float2* dst = a.tf + (t * a.n_kinds * a.Z) * (long long)a.Y * Xh + rem * Xh;  // slot 0 of this row
 
   constexpr bool DZ = MODE >= 1;
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kPsfThreads, 4) k_psf_rows_pair(TfArgs a) {
     }
   }
 #endif
-  const int kxm0 = a.counts[4 * t0 + 2], kxm1 = a.counts[4 * t1 + 2];
+  const int kxm0 = a.counts[kCounts * t0 + kCntKx], kxm1 = a.counts[kCounts * t1 + kCntKx];
   float2* dst0 = a.tf + (t0 * a.n_kinds * a.Z) * (long long)a.Y * Xh + rem0 * Xh;
   float2* dst1 = a.tf + (t1 * a.n_kinds * a.Z) * (long long)a.Y * Xh + rem1 * Xh;
 

@@ -165,6 +165,18 @@ __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
     double r = 0.0;
     if (a.lf_props > 0) r = a.smooth ? 2.0 * o.na_det : o.na_det + fmin(o.na_det, o.na_ill + tilt);
     if (a.want_fl) r = fmax(r, 2.0 * o.na_det);
+    // the columns the source reaches: |k_x / (X p) - t_x / lambda| <= NA_ill / lambda, one column of margin
+    const double px = (double)X * o.pixel_um;
+    const int half = X / 2;
+    int lo = -half, hi = half;
+    if (!a.smooth) {
+      lo = max(lo, (int)floor((cst[2] - cst[3]) * px) - 1);
+      hi = min(hi, (int)ceil((cst[2] + cst[3]) * px) + 1);
+    }
+    int* cnt = a.counts + kCounts * t;
+    cnt[kCntLo] = lo;
+    cnt[kCntHi] = hi;
+    cnt[kCntAxial] = (o.tilt_x == 0.0 && o.tilt_y == 0.0) ? 1 : 0;
     a.stats[(long long)t * 8 + 5] = (float)(r / o.lambda_um * o.pixel_um + 2.0 / (double)min(Y, X));
   }
   const double px = __dmul_rn((double)X, o.pixel_um), py = __dmul_rn((double)Y, o.pixel_um);
@@ -193,7 +205,7 @@ __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
   const float rsf = (float)rs, lamf = (float)lam;
   const float inv_rp = (float)cst[6];  // unit-pupil coordinates of the aberration
   const float wedge = (float)cst[7];
-  int n_sp = 0, n_p = 0, kx_band = -1;
+  int n_sp = 0, n_p = 0, kx_band = -1, ky_band = -1;
   float s_sp = 0.f, s_tx = 0.f, s_ty = 0.f, s_na = 0.f;
   const int rows = min(kRecRows, Y - y0);
   for (int e = threadIdx.x; e < rows * X; e += 256) {
@@ -264,22 +276,25 @@ __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
     // contained in nu_x^2 <= (NA_det/lambda)^2, so every column beyond it is
     // zero in every arm.
     if (y0 + yy == 0 && P) kx_band = max(kx_band, abs(fft_index(x, X)));
+    if (x == 0 && P) ky_band = max(ky_band, abs(fft_index(y0 + yy, Y)));
   }
   for (int off = 16; off > 0; off >>= 1) {
     n_sp += __shfl_down_sync(0xffffffffu, n_sp, off);
     n_p += __shfl_down_sync(0xffffffffu, n_p, off);
     kx_band = max(kx_band, __shfl_down_sync(0xffffffffu, kx_band, off));
+    ky_band = max(ky_band, __shfl_down_sync(0xffffffffu, ky_band, off));
     s_sp += __shfl_down_sync(0xffffffffu, s_sp, off);
     s_tx += __shfl_down_sync(0xffffffffu, s_tx, off);
     s_ty += __shfl_down_sync(0xffffffffu, s_ty, off);
     s_na += __shfl_down_sync(0xffffffffu, s_na, off);
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ int band[8];
+  __shared__ int band[8], bandy[8];
   if (lane == 0) {
     part[0][warp] = n_sp;
     part[1][warp] = n_p;
     band[warp] = kx_band;
+    bandy[warp] = ky_band;
     fpart[0][warp] = s_sp;
     fpart[1][warp] = s_tx;
     fpart[2][warp] = s_ty;
@@ -287,15 +302,18 @@ __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int ca = 0, cb = 0, k = -1;
+    int ca = 0, cb = 0, k = -1, ky = -1;
     for (int i = 0; i < 8; ++i) {
+      ky = max(ky, bandy[i]);
       ca += part[0][i];
       cb += part[1][i];
       k = max(k, band[i]);
     }
-    if (ca) atomicAdd(&a.counts[4 * t], ca);
-    if (cb) atomicAdd(&a.counts[4 * t + 1], cb);
-    if (k >= 0) atomicMax(&a.counts[4 * t + 2], k);
+    int* cnt = a.counts + kCounts * t;
+    if (ca) atomicAdd(cnt + kCntSP, ca);
+    if (cb) atomicAdd(cnt + kCntP, cb);
+    if (k >= 0) atomicMax(cnt + kCntKx, k);
+    if (ky >= 0) atomicMax(cnt + kCntKy, ky);
   }
   // smooth source: per-block partial sums, reduced per tile in a fixed order
   if (a.smooth && threadIdx.x < 4) {
@@ -332,7 +350,7 @@ __global__ void __launch_bounds__(ColGeom<N>::NT, (1024 / ColGeom<N>::NT) > 1 ? 
   const int w = min(B, X - x0);
   // skip strips whose columns all lie outside the detection band: every arm
   // is exactly zero there, and the row pass never reads those columns
-  const int kxmax = a.counts[4 * t + 2];
+  const int kxmax = a.counts[kCounts * t + kCntKx];
   bool active = false;
   for (int b = 0; b < w; ++b) active |= abs(fft_index(x0 + b, X)) <= kxmax;
   if (!active) return;  // uniform across the CTA
@@ -482,7 +500,7 @@ __global__ void __launch_bounds__(PsfGeom<NX>::NT, PsfGeom<NX>::MINB) k_psf_rows
     const int t = (int)((row < nrows ? row : nrows - 1) / ((long long)a.Z * a.Y));
     sc[threadIdx.x] = lf_scale(a, t);
     sc[B + threadIdx.x] = fl_scale(a, t);
-    kxm[threadIdx.x] = row < nrows ? a.counts[4 * t + 2] : -1;
+    kxm[threadIdx.x] = row < nrows ? a.counts[kCounts * t + kCntKx] : -1;
   }
   __syncthreads();
   const long long plane_elems = (long long)a.Y * NX;
@@ -663,6 +681,7 @@ static cudaError_t launch_arms(const TfArgs& a, cudaStream_t s) {
 }
 
 cudaError_t tf_arms(const TfArgs& a, cudaStream_t s) {
+  if (tf_even_supported(a)) return tf_arms_even(a, s);
   if (arms_reg_supported(a.Y, a)) return tf_arms_reg(a, s);
   switch (a.Y) {
 #define WO_CASE(n) \
@@ -694,6 +713,7 @@ static cudaError_t launch_psf(const TfArgs& a, cudaStream_t s) {
 }
 
 cudaError_t tf_psf_rows(const TfArgs& a, cudaStream_t s) {
+  if (tf_even_supported(a)) return tf_psf_rows_even(a, s);
   if (psf_rows_reg_supported(a.X, a.n_arms)) return tf_psf_rows_reg(a, s);
   switch (a.X) {
 #define WO_CASE(n) \

@@ -6,11 +6,18 @@ namespace wo {
 
 __device__ __forceinline__ int fft_index(int i, int n) { return (i < (n + 1) / 2) ? i : i - n; }
 
+// Per-tile words of the pupil record (TfArgs::counts, kCounts ints per tile,
+// zeroed before the record kernel): #(S and P) of a binary source, #P, the
+// largest |k_x| and |k_y| inside P, the range of k_x the source reaches inside
+// P (conservative; the whole band for a smooth source), 1 when the
+// illumination is on axis (S depends on |k_x| and |k_y| alone).
+enum { kCntSP = 0, kCntP = 1, kCntKx = 2, kCntKy = 3, kCntLo = 4, kCntHi = 5, kCntAxial = 6 };
+
 __device__ __forceinline__ float lf_scale(const TfArgs& a, int t) {
   // 2K = 2 c / (N_perp sum S P^2), c = 2 pi n dz / lambda^2; the sum is a count
   // for the binary source and a float sum for the smooth one
   const wo_optics o = a.optics[t];
-  const double sp = a.smooth ? (double)a.norms[4 * t] : (double)a.counts[4 * t];
+  const double sp = a.smooth ? (double)a.norms[4 * t] : (double)a.counts[kCounts * t + kCntSP];
   if (!(sp > 0.0)) return 0.f;
   const double c = 2.0 * 3.14159265358979323846 * o.n_medium * o.z_step_um / (o.lambda_um * o.lambda_um);
   return (float)(2.0 * c / ((double)a.Y * (double)a.X * sp));
@@ -24,7 +31,7 @@ __device__ __forceinline__ float norm_dlog(const TfArgs& a, int t, int theta) {
 }
 
 __device__ __forceinline__ float fl_scale(const TfArgs& a, int t) {
-  const int n_p = a.counts[4 * t + 1];
+  const int n_p = a.counts[kCounts * t + kCntP];
   if (n_p == 0) return 0.f;
   return (float)(1.0 / ((double)a.Y * (double)a.X * (double)a.Z * (double)n_p));
 }
