@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4)
 #pragma unroll
       for (int m = 0; m < N1; ++m) w[m] = cscale(cmulc(va[m], vb[m]), sc);
     }
-    P::template fft<false>(w, tw, S, lt);
+    P::template fft<false, (DZ ? 1 : 0)>(w, tw, S, lt);
 #pragma unroll
     for (int m = 0; m < N1; ++m) {
       const float2 mv = mirror_value<N1>(w, m, lane0);
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4)
     P::template fft<true>(vs, tw, S, lt);
 #pragma unroll
     for (int m = 0; m < N1; ++m) w[m].y = sc * (vs[m].x * vb[m].x + vs[m].y * vb[m].y - ry * gre[m]);
-    P::template fft<false>(w, tw, S, lt);
+    P::template fft<false, (DZ ? 1 : 0)>(w, tw, S, lt);
 #pragma unroll
     for (int m = 0; m < N1; ++m) {
       const float2 mv = mirror_value<N1>(w, m, lane0);
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4)
     P::template fft<true>(vs, tw, S, lt);
 #pragma unroll
     for (int m = 0; m < N1; ++m) w[m] = make_float2(sc * (vs[m].x * vb[m].x + vs[m].y * vb[m].y - rn * gre[m]), 0.f);
-    P::template fft<false>(w, tw, S, lt);
+    P::template fft<false, 2>(w, tw, S, lt);
 #pragma unroll
     for (int m = 0; m < N1; ++m) {
       const int k = lt + T * m;
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4)
     P::template fft<true>(w, tw, S, lt);
 #pragma unroll
     for (int m = 0; m < N1; ++m) w[m] = make_float2(scf * cabs2(w[m]), 0.f);
-    P::template fft<false>(w, tw, S, lt);
+    P::template fft<false, (DZ ? 1 : 0)>(w, tw, S, lt);
 #pragma unroll
     for (int m = 0; m < N1; ++m) {
       const int k = lt + T * m;

@@ -67,8 +67,11 @@ __device__ __forceinline__ float2 twiddle_mul(float2 a, int e) {
   return cmul(a, make_float2(kW48.re[m], INV ? -kW48.im[m] : kW48.im[m]));
 }
 
-// In-register Stockham stages over L points (natural order in and out).
-template <int L, int NS, bool INV, int STEP>
+// In-register Stockham stages over L points (natural order in and out).  SC
+// > 0: the first stage in scalar form (its inputs are products, see dftR);
+// SC > 1: every stage (a real row, whose twiddle products are single
+// products too).
+template <int L, int NS, bool INV, int STEP, int SC = 0>
 __device__ __forceinline__ void reg_stages(float2 (&v)[L], const float2* tw) {
   if constexpr (NS < L) {
     constexpr int R = radix_for(L / NS);
@@ -84,14 +87,14 @@ __device__ __forceinline__ void reg_stages(float2 (&v)[L], const float2* tw) {
 #pragma unroll
         for (int r = 1; r < R; ++r) w[r] = twiddle_mul<INV, NS * R>(w[r], r * k);
       }
-      dftR<R, INV>(w);
+      dftR<R, INV, (SC > 1 || (SC == 1 && NS == 1))>(w);
       const int base = (j / NS) * NS * R + k;
 #pragma unroll
       for (int r = 0; r < R; ++r) o[base + r * NS] = w[r];
     }
 #pragma unroll
     for (int i = 0; i < L; ++i) v[i] = o[i];
-    reg_stages<L, NS * R, INV, STEP>(v, tw);
+    reg_stages<L, NS * R, INV, STEP, SC>(v, tw);
   }
 }
 
@@ -118,9 +121,9 @@ struct Row2 {
     }
   }
 
-  template <bool INV>
+  template <bool INV, int SC = 0>
   static __device__ __forceinline__ void fft(float2 (&v)[E], const float2* tw, float2* S, int t) {
-    reg_stages<N1, 1, INV, N / N1>(v, tw);
+    reg_stages<N1, 1, INV, N / N1, SC>(v, tw);
 #pragma unroll
     for (int k1 = 1; k1 < N1; ++k1) {
       float2 w = tw[N + k1 * T + t];
@@ -164,10 +167,10 @@ struct Row512 {
     }
   }
 
-  template <bool INV>
+  template <bool INV, int SC = 0>
   static __device__ __forceinline__ void fft(float2 (&v)[E], const float2* tw, float2* S, int l) {
     // pass 1 (sub-length 1, radix 16): butterfly l takes points l + 32 r
-    reg_stages<16, 1, INV, 32>(v, tw);
+    reg_stages<16, 1, INV, 32, SC>(v, tw);
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < 16; ++r) S[pad(16 * l + r)] = v[r];
