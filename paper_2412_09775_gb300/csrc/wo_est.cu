@@ -55,66 +55,127 @@ __device__ __forceinline__ float bf(const __nv_bfloat16* p, long long i) { retur
 // ---------------------------------------------------------------- features
 __device__ __forceinline__ int freq_idx(int i, int n) { return (i < (n + 1) / 2) ? i : i - n; }
 
-// One block per (natural row r, tile): radial sums of the plane's power and of
+// One warp per (natural row r, tile): radial sums of the plane's power and of
 // the cross spectrum with the next plane, over the half spectrum with the
 // weights of the conjugate pairs.  Rows >= Z are zero.  ch0 holds the raw
 // power until k_feat_norm.
-__global__ void __launch_bounds__(256) k_features(const float2* __restrict__ spec, const wo_optics* __restrict__ optics,
-                                                  int Z, int Y, int X, float* __restrict__ feat) {
-  __shared__ float P[kSide], den[kSide], sx[kSide], sy[kSide];
-  const int r = blockIdx.x, t = blockIdx.y;
+//
+// Shared-memory float atomics bounded the former kernel (four a point, and
+// the neighbours of a ring meet in one bin).  Here two lanes of a warp share
+// 64 bins of {P, den, sx, sy} and add to them in turn (16 KB a warp; a slot
+// keeps its own banks whatever the bin), so a point costs one 16-byte load and
+// store and no atomic; the slots are summed at the end, in a fixed order.  The
+// rows y and Y - y of a plane share their frequencies' geometry and bin and
+// are added together.  Four warps take four rows r of one tile: the geometry
+// of 128 points at a time is formed once for them, and a warp's next plane is
+// its neighbour's plane (L1 hits).  Four points of a lane have their loads in
+// flight at once.  256 x 48x128x128: 1374 -> 616 us (one warp a CTA with a
+// slot a lane, the geometry formed by every warp: about 945 us).
+constexpr int kFeatRows = 4, kFeatPts = 32 * kFeatRows, kFeatSlots = 16;
+
+__global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict__ spec,
+                                                       const wo_optics* __restrict__ optics, int Z, int Y, int X,
+                                                       float* __restrict__ feat) {
+  extern __shared__ float4 sm4[];
+  float4* geo = sm4;                                                      // [2][128]: ux, uy, w, bin (-1: none)
+  int2* off = reinterpret_cast<int2*>(geo + 2 * kFeatPts);                // [2][128]: the points at y and Y - y (-1: none)
+  const int wi = threadIdx.x / 32, lane = threadIdx.x & 31;
+  float4* bins = reinterpret_cast<float4*>(off + 2 * kFeatPts) + wi * kSide * kFeatSlots;  // [64][16]
+  const int r = blockIdx.x * kFeatRows + wi, t = blockIdx.y;
   const int Xh = X / 2 + 1;
-  for (int i = threadIdx.x; i < kSide; i += blockDim.x) P[i] = den[i] = sx[i] = sy[i] = 0.f;
-  __syncthreads();
-  float* out = feat + (long long)t * 3 * kSide * kSide + (long long)r * kSide;
-  if (r < Z) {
-    const wo_optics o = optics[t];
-    const double cut = 2.0 * o.na_det / o.lambda_um;
-    const long long plane = (long long)Y * Xh;
-    const float2* Dr = spec + ((long long)t * Z + ((r - Z / 2 + Z) % Z)) * plane;
-    const bool nxt = r + 1 < Z;
-    const float2* Dn = spec + ((long long)t * Z + ((r + 1 - Z / 2 + Z) % Z)) * plane;
-    // the radial bin is decided in float where the value is clear of a bin
-    // edge by far more than the float error (relative 3e-7 of at most 64),
-    // and by the float64 expression otherwise, so the bins equal the
-    // float64 ones (float64 is slow on this part)
-    const float inv_py = (float)(1.0 / ((double)Y * o.pixel_um)), inv_px = (float)(1.0 / ((double)X * o.pixel_um));
-    const float qscale = (float)((double)kSide / cut);
-    for (long long e = threadIdx.x; e < plane; e += blockDim.x) {
-      const int y = (int)(e / Xh), x = (int)(e - (long long)y * Xh);
-      const float fyf = (float)freq_idx(y, Y) * inv_py, fxf = (float)x * inv_px;
-      const float radf = sqrtf(fxf * fxf + fyf * fyf);
-      const float q = radf * qscale;
-      const float fr = q - floorf(q);
-      int b;
-      if (fr > 1e-4f && fr < 1.f - 1e-4f) {
-        b = (int)floorf(q);
-      } else {
-        const double fy = (double)freq_idx(y, Y) / ((double)Y * o.pixel_um);
-        const double fx = (double)x / ((double)X * o.pixel_um);
-        b = (int)floor(sqrt(fx * fx + fy * fy) / cut * kSide);
+  const double pixel = optics[t].pixel_um, cut = 2.0 * optics[t].na_det / optics[t].lambda_um;
+  for (int b = lane; b < kSide * kFeatSlots; b += 32) bins[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const long long plane = (long long)Y * Xh;
+  const bool row = r < Z, nxt = r + 1 < Z;
+  const float2* Dr = spec + ((long long)t * Z + (row ? (r - Z / 2 + Z) % Z : 0)) * plane;
+  // the last row has no next plane: it reads its own and leaves den, sx, sy out
+  const float2* Dn = nxt ? spec + ((long long)t * Z + ((r + 1 - Z / 2 + Z) % Z)) * plane : Dr;
+  // the radial bin is decided in float where the value is clear of a bin
+  // edge by far more than the float error (relative 4e-7 of at most 64),
+  // and by the float64 expression otherwise, so the bins equal the
+  // float64 ones (float64 is slow on this part)
+  const float inv_py = (float)(1.0 / ((double)Y * pixel)), inv_px = (float)(1.0 / ((double)X * pixel));
+  const float qscale = (float)((double)kSide / cut);
+  const int points = (Y / 2 + 1) * Xh;
+  for (int p0 = 0, buf = 0; p0 < points; p0 += kFeatPts, buf ^= 1) {
+    {
+      const int p = p0 + threadIdx.x;
+      const int y = p / Xh, x = p - y * Xh;
+      const float fy = (float)freq_idx(y, Y) * inv_py, fx = (float)x * inv_px;
+      const float rad = sqrtf(fx * fx + fy * fy);
+      const float q = rad * qscale, fl = floorf(q), fr = q - fl;
+      int b = (int)fl;
+      if (p < points && !(fr > 1e-4f && fr < 1.f - 1e-4f)) {
+        const double gy = (double)freq_idx(y, Y) / ((double)Y * pixel);
+        const double gx = (double)x / ((double)X * pixel);
+        b = (int)floor(sqrt(gx * gx + gy * gy) / cut * kSide);
       }
-      if (b >= kSide) continue;
-      const float w = (x == 0 || 2 * x == X) ? 1.f : 2.f;
-      const float2 dr = Dr[e];
-      atomicAdd(&P[b], w * cabs2(dr));
+      if (p >= points || b >= kSide) b = -1;
+      geo[buf * kFeatPts + threadIdx.x] =
+          make_float4(rad > 0.f ? fx / rad : 0.f, rad > 0.f ? fy / rad : 0.f, (x == 0 || 2 * x == X) ? 1.f : 2.f,
+                      __int_as_float(b));
+      off[buf * kFeatPts + threadIdx.x] = make_int2(y * Xh + x, (y > 0 && 2 * y < Y) ? (Y - y) * Xh + x : -1);
+    }
+    __syncthreads();  // (the other buffer's readers are past their loop)
+    if (!row) continue;
+    float2 dr[kFeatRows], dn[kFeatRows], mr[kFeatRows], mn[kFeatRows];
+    float4 g[kFeatRows];
+    const float2 zero = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kFeatRows; ++i) {
+      g[i] = geo[buf * kFeatPts + 32 * i + lane];
+      const int2 o = off[buf * kFeatPts + 32 * i + lane];
+      const bool on = __float_as_int(g[i].w) >= 0, two = on && o.y >= 0;
+      dr[i] = on ? __ldg(Dr + o.x) : zero;
+      dn[i] = on ? __ldg(Dn + o.x) : zero;
+      mr[i] = two ? __ldg(Dr + o.y) : zero;
+      mn[i] = two ? __ldg(Dn + o.y) : zero;
+    }
+#pragma unroll
+    for (int i = 0; i < kFeatRows; ++i) {
+      const int b = __float_as_int(g[i].w);
+      const float pr = cabs2(dr[i]), pm = cabs2(mr[i]);
+      // Im of D_next conj(D_r), at y and Y - y
+      const float ci = dr[i].x * dn[i].y - dr[i].y * dn[i].x, cm = mr[i].x * mn[i].y - mr[i].y * mn[i].x;
+      const float w = g[i].z;
+      float4 v = make_float4(w * (pr + pm), 0.f, 0.f, 0.f);
       if (nxt) {
-        const float2 dn = Dn[e];
-        const float2 c = cmulc(dr, dn);  // dn * conj(dr)
-        const float ux = radf > 0.f ? fxf / radf : 0.f, uy = radf > 0.f ? fyf / radf : 0.f;
-        atomicAdd(&den[b], w * sqrtf(cabs2(dn) * cabs2(dr)));
-        atomicAdd(&sx[b], w * c.y * ux);
-        atomicAdd(&sy[b], w * c.y * uy);
+        v.y = w * (sqrtf(cabs2(dn[i]) * pr) + sqrtf(cabs2(mn[i]) * pm));
+        v.z = w * (ci + cm) * g[i].x;
+        v.w = w * (ci - cm) * g[i].y;
+      }
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {  // the slot's two lanes in turn
+        if (b >= 0 && lane / kFeatSlots == half) {
+          float4& s = bins[b * kFeatSlots + (lane & (kFeatSlots - 1))];
+          const float4 u = s;
+          s = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
+        }
+        __syncwarp();
       }
     }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kSide; i += blockDim.x) {
-    out[i] = P[i];
-    out[kSide * kSide + i] = den[i] > 0.f ? sx[i] / den[i] : 0.f;
-    out[2 * kSide * kSide + i] = den[i] > 0.f ? sy[i] / den[i] : 0.f;
+  if (r >= kSide) return;
+  float* out = feat + (long long)t * 3 * kSide * kSide + (long long)r * kSide;
+  __syncwarp();
+  for (int b = lane; b < kSide; b += 32) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int l = 0; l < kFeatSlots; ++l) {  // each lane starts at another slot: distinct banks
+      const float4 u = bins[b * kFeatSlots + ((l + lane) & (kFeatSlots - 1))];
+      v.x += u.x;
+      v.y += u.y;
+      v.z += u.z;
+      v.w += u.w;
+    }
+    out[b] = v.x;
+    out[kSide * kSide + b] = v.y > 0.f ? v.z / v.y : 0.f;
+    out[2 * kSide * kSide + b] = v.y > 0.f ? v.w / v.y : 0.f;
   }
 }
+
+constexpr size_t kFeatSmem = 2 * kFeatPts * (sizeof(float4) + sizeof(int2)) +
+                             (size_t)kFeatRows * kSide * kFeatSlots * sizeof(float4);
 
 // One block per tile: ch0 = log(1 + P / mean P) over the Z valid rows.
 __global__ void __launch_bounds__(256) k_feat_norm(int Z, float* __restrict__ feat) {
@@ -380,9 +441,11 @@ size_t est_workspace_bytes(int B) { return est_ws(B).total; }
 
 cudaError_t est_features(const float2* spec, const wo_optics* optics, int n, int Z, int Y, int X, float* feat,
                          cudaStream_t s) {
-  dim3 grid((unsigned)kSide, (unsigned)n);
-  WO_LAUNCH("est_features", s, (k_features<<<grid, 256, 0, s>>>(spec, optics, Z, Y, X, feat)));
-  cudaError_t e = cudaGetLastError();
+  dim3 grid((unsigned)(kSide / kFeatRows), (unsigned)n);
+  cudaError_t e = allow_smem(k_features, kFeatSmem);
+  if (e != cudaSuccess) return e;
+  WO_LAUNCH("est_features", s, (k_features<<<grid, kFeatPts, kFeatSmem, s>>>(spec, optics, Z, Y, X, feat)));
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   WO_LAUNCH("est_feat_norm", s, (k_feat_norm<<<(unsigned)n, 256, 0, s>>>(Z, feat)));
   return cudaGetLastError();
