@@ -66,10 +66,10 @@ CPU_SAMPLE = (96, 256, 256)
 # capture), scaled by 4 to the 256 tiles of a launch of the bench's field
 # (the traffic grows with the tiles).
 NCU_TRAFFIC = {
-    ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "ecc17f300571f036"},
-    ("field", "tf_psf_rows"): {"bytes": 4 * (584036096 + 423149568), "digest": "e3d455139ebd183f"},
-    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "676ec8236312b6b9"},
-    ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "676ec8236312b6b9"},
+    ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "2c11b6414f8dfa33"},
+    ("field", "tf_psf_rows"): {"bytes": 4 * (584036096 + 423149568), "digest": "6abc643aaa56a40a"},
+    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "5556489b6f389c1b"},
+    ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "5556489b6f389c1b"},
 }
 
 

@@ -272,6 +272,72 @@ __device__ __forceinline__ void fft_smem(float2* buf, int es, int bs, const floa
   fft_smem_a<N, B, NT, INV, TWS>(buf, LinAddr{es, bs}, tw);
 }
 
+// A transform whose first stage takes its inputs from in(n, b, i) (i: the
+// thread's i-th point, a constant) and whose last stage hands its outputs to
+// out(n, b, value): the tile is written to and read
+// from shared memory only between stages.  The arithmetic is fft_smem's.  The
+// caller has the twiddles under way (they are first read behind a barrier
+// here, or not at all), or MAKE_TW has them made while the first inputs are on
+// their way; before buf is written again, it needs a barrier of its own.  Every in() of the CTA comes before any out(), so a tile can be
+// transformed in place in global memory.  N <= 8 is one stage: a thread then
+// reads and writes the same points.
+template <int N, int B, int NT, bool INV, int R, int NS, bool FIRST, bool MAKE_TW, class In, class Out>
+__device__ __forceinline__ void fft_stage_io(float2* buf, float2* tw, int tid, In in, Out out) {
+  constexpr int M = N / R, NB = M * B, PER = (NB + NT - 1) / NT;
+  constexpr bool LAST = NS * R == N;
+  // the last stage may go one butterfly at a time: nothing is written back
+  constexpr int G = LAST ? 1 : PER;
+#pragma unroll
+  for (int i0 = 0; i0 < PER; i0 += G) {
+    float2 v[G][R];
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const int beta = tid + (i0 + i) * NT;
+      if ((NB % NT == 0) || beta < NB) {
+        const int b = beta % B, j = beta / B;
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[i][r] = FIRST ? in(j + r * M, b, (i0 + i) * R + r) : buf[(j + r * M) * B + b];
+      }
+    }
+    if (MAKE_TW && i0 == 0) make_twiddles<N>(tw);
+    if (!FIRST && !LAST) __syncthreads();
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      const int beta = tid + (i0 + i) * NT;
+      if ((NB % NT == 0) || beta < NB) {
+        const int b = beta % B, j = beta / B;
+        const int k = j % NS;
+        if constexpr (NS > 1) {
+          constexpr int STEP = N / (NS * R);
+#pragma unroll
+          for (int r = 1; r < R; ++r) {
+            float2 w = tw[r * k * STEP];
+            if (INV) w.y = -w.y;
+            v[i][r] = cmul(v[i][r], w);
+          }
+        }
+        dftR<R, INV>(v[i]);
+        const int base = (j / NS) * NS * R + k;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if constexpr (LAST) out(base + r * NS, b, v[i][r]);
+          else buf[(base + r * NS) * B + b] = v[i][r];
+        }
+      }
+    }
+  }
+  if (!LAST) __syncthreads();
+}
+
+template <int N, int B, int NT, bool INV, bool MAKE_TW, class In, class Out, int NS = 1>
+__device__ __forceinline__ void fft_through(float2* buf, float2* tw, int tid, In in, Out out) {
+  if constexpr (NS < N) {
+    constexpr int R = radix_for(N / NS);
+    fft_stage_io<N, B, NT, INV, R, NS, NS == 1, MAKE_TW && NS == 1 && (R < N)>(buf, tw, tid, in, out);
+    fft_through<N, B, NT, INV, MAKE_TW, In, Out, NS * R>(buf, tw, tid, in, out);
+  }
+}
+
 // ------------------------------------------------------------ async copies
 // cp.async (global -> shared, bypassing registers): a thread issues all of its
 // copies before waiting, so a whole tile is in flight at once.  A source size

@@ -1,0 +1,45 @@
+"""The column, row and z passes at the lengths and edges where their kernels
+differ, against the same step in float64 torch.
+
+Bounds: a float32 transform of a few thousand points is a few 1e-7 off its
+exact value (relative 2-norm); an operator is two three-dimensional ones and
+a product, about 1e-6; both are allowed five times that.
+"""
+import numpy as np
+import pytest
+
+import phantom as ph
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    from paper_2412_09775_gb300.build import build
+    build()
+    from paper_2412_09775_gb300 import binding
+    return binding, torch, torch.device("cuda:0")
+
+
+def rel(torch, got, want):
+    dt = torch.complex128 if want.is_complex() else torch.float64
+    return float(torch.linalg.vector_norm(got.to(dt) - want) / torch.linalg.vector_norm(want))
+
+
+def noise(torch, dev, seed, *shape):
+    g = torch.Generator(device=dev)
+    g.manual_seed(seed)
+    return torch.randn(shape, generator=g, device=dev)
+
+
+@pytest.mark.parametrize("Y", [2, 3, 6, 8, 12, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 2048])
+@pytest.mark.parametrize("X", [2, 96])
+def test_plane_spectra_at_every_column_length(env, Y, X):
+    """Columns of one to four stages, strips of one, 16 and a last odd column."""
+    B, torch, dev = env
+    d = noise(torch, dev, Y, 2, 3, Y, X)
+    spec = torch.empty((2, 3, Y, X // 2 + 1), dtype=torch.complex64, device=dev)
+    B.wo_spectrum(d, [0.0], B.WO_MODE_2D, spec, 2, 3, Y, X)
+    assert rel(torch, spec, torch.fft.rfft2(d.double())) < 1.5e-6
