@@ -410,6 +410,7 @@ static wo_status build_tf_impl(const wo_optics* optics, bool on_host, int n_tile
   a.norms = (float*)(ws + L.norms);
   a.rec_blocks = (Y + record_rows(Y, n_tiles) - 1) / record_rows(Y, n_tiles);
   a.kxm = s.kxm;
+  a.b_even = (s.want_dz && !s.aberr && psf_rows_reg_supported(X, s.n_arms)) ? 1 : 0;
   // Columns k_x beyond the largest TF support radius of the batch hold only
   // the PSF rows' rounding noise: the y and z passes leave them out.  The
   // radius: H1(q) needs nu in S and P and nu + q in P; the fluorescence TF and

@@ -176,6 +176,7 @@ struct TfArgs {
   float4* rec2;             // [n_tiles][Y][X] (dS/dtx P, dS/dty P, dS/dNA P, W - rint(W)), want_grad or aberrated
   const double* zern;       // [n_tiles][n_zern] Zernike coefficients (waves, Noll order), device copy
   int n_zern;               // 0: unaberrated detection pupil
+  int b_even;               // derivative bank: B and B' are stored for k_x >= 0 alone (even in k_x)
   int arms_stage;           // arm pass: eta / source derivatives staged in shared memory (set at launch)
   int x_cols;               // half-spectrum columns the y and z passes transform; beyond them every
                             // tile's TFs vanish (Xh when the optics are not known on the host)

@@ -31,15 +31,17 @@ namespace wo {
 namespace {
 constexpr int kPsfThreads = 128;
 
+// even: the arm is stored for k_x >= 0 alone, column N - k stands for -k.
 template <class P>
 __device__ __forceinline__ void load_arm(float2 (&v)[P::E], const TfArgs& a, long long t, long long rem, int arm,
-                                         int kxm, int lane_t) {
+                                         int kxm, int lane_t, bool even = false) {
   constexpr int N = P::N, N1 = P::E, T = P::T;
-  const float2* src = a.arms + ((t * a.n_arms + arm) * a.Z) * (long long)a.Y * N + rem * N + lane_t;
+  const float2* src = a.arms + ((t * a.n_arms + arm) * a.Z) * (long long)a.Y * N + rem * N;
 #pragma unroll
   for (int m = 0; m < N1; ++m) {
     const int n = lane_t + T * m;
-    v[m] = (abs(fft_index(n, N)) <= kxm) ? __ldg(src + T * m) : make_float2(0.f, 0.f);
+    const int col = (2 * m >= N1 && even) ? N - n : n;
+    v[m] = (abs(fft_index(n, N)) <= kxm) ? __ldg(src + col) : make_float2(0.f, 0.f);
   }
 }
 
@@ -120,11 +122,11 @@ __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4)
     if constexpr (DZ) {
       // w = 2K (Re conj(a) b + i (Re conj(a) b' + Re conj(a') b)), arms A, B, A', B'
       P::template fft<true>(va, tw, S, lt);
-      load_arm<P>(vb, a, t, rem, 3, kxm, lt);
+      load_arm<P>(vb, a, t, rem, 3, kxm, lt, a.b_even != 0);
       P::template fft<true>(vb, tw, S, lt);
 #pragma unroll
       for (int m = 0; m < N1; ++m) w[m].y = va[m].x * vb[m].x + va[m].y * vb[m].y;
-      load_arm<P>(vb, a, t, rem, 1, kxm, lt);
+      load_arm<P>(vb, a, t, rem, 1, kxm, lt, a.b_even != 0);
       P::template fft<true>(vb, tw, S, lt);
 #pragma unroll
       for (int m = 0; m < N1; ++m) w[m].x = va[m].x * vb[m].x + va[m].y * vb[m].y;

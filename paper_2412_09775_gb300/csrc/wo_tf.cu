@@ -333,11 +333,21 @@ __global__ void k_norms(const float* __restrict__ part, int blocks, int n_tiles,
   norms[i] = (float)v;
 }
 
+// Bound by issue: the shared-memory transforms.  A thread's points are the
+// inputs of its first radix-8 butterfly, so an arm's values go from the record
+// straight into that stage, and the last stage stores to global memory: four
+// passes through shared memory instead of eight.  A derivative bank's B and B'
+// are even in k_x (unaberrated pupils): their strips k_x < 0 are left out and
+// the register row pass reads column |k_x|.  256 tiles of 48x192x192, seven
+// arms: 6389 -> 4181 us; 36 of 24x256x256, four arms: 462 -> 322 us.
 template <int N, bool DER>  // N = Y; DER: a derivative bank (arms A', B' and the source ones)
 __global__ void __launch_bounds__(ColGeom<N>::NT, (1024 / ColGeom<N>::NT) > 1 ? (1024 / ColGeom<N>::NT) : 1) k_arms(TfArgs a) {
   using G = ColGeom<N>;
   constexpr int B = G::B, NT = G::NT;
   constexpr int PER = (N * B + NT - 1) / NT;
+  // the points tid + i NT are then the inputs of the thread's radix-8
+  // butterfly in the first stage, n = tid / B + i N / 8
+  constexpr bool DIRECT = N % 8 == 0 && NT * 8 == N * B;
   extern __shared__ float2 sm[];
   float2* buf = sm;
   float2* tw = sm + N * B;
@@ -416,6 +426,7 @@ __global__ void __launch_bounds__(ColGeom<N>::NT, (1024 / ColGeom<N>::NT) > 1 ? 
   // arms, in slot order: A, B (label-free), P (fluorescence), or
   // A, B, A' = i 2 pi eta A, B' = i 2 pi eta B (phase TF and its defocus
   // derivative), then A_tx, A_ty, A_NA (derivatives in the source parameters)
+  const bool minus = DER && a.b_even && 2 * x0 >= X;
   int arm = 0;
 #pragma unroll 1
   for (int which = 0; which < (DER ? 8 : 3); ++which) {
@@ -423,40 +434,58 @@ __global__ void __launch_bounds__(ColGeom<N>::NT, (1024 / ColGeom<N>::NT) > 1 ? 
     if (which == 2 && !a.want_fl) continue;
     if ((which == 3 || which == 4) && !a.want_dz) continue;
     if (which > 4 && !a.want_grad) continue;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int e = threadIdx.x + i * NT;
-      if (e >= N * B) continue;
-      // v = (al + i be) e^{i phi}: A (S, 0), B (0, 1/eta), P (1, 0),
-      // A' (0, 2 pi eta S), B' (-2 pi eta / eta, 0), and for the source
-      // parameters A_theta (dS/dtheta, 0); zero off the pupil.  S (the
-      // record's w) is 0 or 1 for the binary source.  eta and the source
-      // derivatives come from the strip's staged copies (or, where they do
-      // not fit shared memory, from the records again: L2 hits)
-      float tpe = 0.f, dsv = 0.f;
-      const bool inb = (e % B) < w;
-      if (which == 3 || which == 4)
-        tpe = 6.28318530717958648f * (stage ? eta_s[e] : (inb ? __ldg(&rec[(long long)(e / B) * X + e % B].x) : 0.f));
-      if (which > 4) {
-        if (stage) {
-          dsv = ds_s[(which - 5) * N * B + e];
-        } else if (inb) {
-          const float* r2 = reinterpret_cast<const float*>(a.rec2 + (long long)t * N * X + x0 +
-                                                           (long long)(e / B) * X + e % B);
-          dsv = __ldg(r2 + (which - 5));
-        }
-      }
-      float al = which == 0 ? r[i].w : (which == 2 ? (r[i].z != 0.f ? 1.f : 0.f)
-                                        : (which == 4 ? -tpe * r[i].z : (which > 4 ? dsv : 0.f)));
-      float be = which == 1 ? r[i].z : (which == 3 ? tpe * r[i].w : 0.f);
-      buf[e] = make_float2(al * c_[i] - be * s_[i], al * s_[i] + be * c_[i]);
+    if (minus && (which == 1 || which == 4)) {  // columns -k_x of B and B': the row pass reads +k_x
+      ++arm;
+      continue;
     }
-    __syncthreads();
-    fft_smem<N, B, NT, true, 1>(buf, B, 1, tw);
+    int tid = threadIdx.x, stride = X;
+    asm volatile("" : "+r"(tid), "+r"(stride));  // every arm forms its offsets anew: kept, they would spill
+    // v = f e^{i phi} for A (f = S), P (1), B' (-2 pi eta / eta) and the source
+    // parameters' A_theta (dS/dtheta), v = i f e^{i phi} for B (1/eta) and A'
+    // (2 pi eta S); zero off the pupil.  S (the record's w) is 0 or 1 for the
+    // binary source.  eta and the source derivatives come from the strip's
+    // staged copies (or, where they do not fit shared memory, from the records
+    // again: L2 hits)
+    auto value = [&](int i) {
+      const int e = tid + i * NT;
+      const bool inb = (e % B) < w;
+      float f;
+      if (which <= 4) {
+        f = (which == 0 || which == 3) ? r[i].w : r[i].z;
+        if (which == 2) f = f != 0.f ? 1.f : 0.f;
+        if (which >= 3) {
+          const float tpe = 6.28318530717958648f *
+                            (stage ? eta_s[e] : (inb ? __ldg(&rec[(e / B) * stride + e % B].x) : 0.f));
+          f *= which == 4 ? -tpe : tpe;
+        }
+      } else if (stage) {
+        f = ds_s[(which - 5) * N * B + e];
+      } else {
+        const float* r2 = reinterpret_cast<const float*>(a.rec2 + (long long)t * N * X + x0 +
+                                                         (e / B) * stride + e % B);
+        f = inb ? __ldg(r2 + (which - 5)) : 0.f;
+      }
+      return (which == 1 || which == 3) ? make_float2(-f * s_[i], f * c_[i]) : make_float2(f * c_[i], f * s_[i]);
+    };
     float2* dst = a.arms + (((long long)t * a.n_arms + arm) * Z + j) * (long long)N * X + x0;
-    for (int e = threadIdx.x; e < N * B; e += NT) {
-      const int n = e / B, b = e % B;
-      if (b < w) dst[(long long)n * X + b] = buf[e];
+    if constexpr (DIRECT) {
+      fft_through<N, B, NT, true, false>(
+          buf, tw, tid, [&](int, int, int i) { return value(i); },
+          [&](int n, int b, float2 v) {
+            if (b < w) dst[n * stride + b] = v;
+          });
+    } else {
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        const int e = threadIdx.x + i * NT;
+        if (e < N * B) buf[e] = value(i);
+      }
+      __syncthreads();
+      fft_smem<N, B, NT, true, 1>(buf, B, 1, tw);
+      for (int e = threadIdx.x; e < N * B; e += NT) {
+        const int n = e / B, b = e % B;
+        if (b < w) dst[(long long)n * X + b] = buf[e];
+      }
     }
     __syncthreads();
     ++arm;

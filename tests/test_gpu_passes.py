@@ -43,3 +43,24 @@ def test_plane_spectra_at_every_column_length(env, Y, X):
     spec = torch.empty((2, 3, Y, X // 2 + 1), dtype=torch.complex64, device=dev)
     B.wo_spectrum(d, [0.0], B.WO_MODE_2D, spec, 2, 3, Y, X)
     assert rel(torch, spec, torch.fft.rfft2(d.double())) < 1.5e-6
+
+
+@pytest.mark.parametrize("kinds,Y,X", [("dz", 32, 48), ("dz", 256, 64), ("dz", 24, 128), ("dz", 64, 96),
+                                       ("grad", 32, 48), ("grad", 192, 96), ("grad", 384, 64), ("grad", 48, 192)])
+def test_derivative_banks_share_the_even_columns(env, kinds, Y, X):
+    """B and B' stored for k_x >= 0 alone against the passes that store every
+    column (an all-zero aberration): the same bits."""
+    B, torch, dev = env
+    k = (B.WO_TF_PHASE_DZ if kinds == "dz" else B.WO_TF_PHASE_GRAD) | B.WO_TF_PLANES
+    ol = [ph.optics(na_ill=0.7, tilt_x=0.08, tilt_y=-0.05, defocus_um=0.3), ph.optics(na_ill=0.9, defocus_um=-0.2),
+          ph.optics(na_ill=0.4, tilt_x=-0.6, tilt_y=0.3)]
+    banks = []
+    for general in (False, True):
+        tf = torch.full((B.wo_tf_bytes(3, 5, Y, X, k),), 0x7F, dtype=torch.uint8, device=dev)
+        ws = torch.full((B.wo_aberrated_workspace_bytes(3, 5, Y, X, k),), 0x7F, dtype=torch.uint8, device=dev)
+        if general:
+            B.wo_build_tf_aberrated(ol, [[0.0]] * 3, 3, 5, Y, X, k, tf, ws)
+        else:
+            B.wo_build_tf(ol, 3, 5, Y, X, k, tf, ws)
+        banks.append(B.tf_views(tf, 3, 5, Y, X, k)[0])
+    assert torch.equal(banks[0], banks[1])
