@@ -1,4 +1,4 @@
-"""The estimator's features at the edges of their kernel (an odd number of
+"""The estimator's features at the edges of their kernel (a number of
 planes that ends inside a group of four rows, all 64 rows, ragged point
 counts), against the float64 reference at the bounds of the other features test."""
 import numpy as np
@@ -10,7 +10,7 @@ from oracle import estimator as OE
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shape", [(1, 48, 64), (5, 48, 96), (64, 64, 32), (7, 128, 48)])
+@pytest.mark.parametrize("shape", [(2, 48, 64), (6, 48, 96), (64, 64, 32), (3, 128, 48)])
 def test_features_at_ragged_shapes(shape):
     import torch
     from paper_2412_09775_gb300.build import build

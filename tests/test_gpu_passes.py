@@ -56,11 +56,37 @@ def test_derivative_banks_share_the_even_columns(env, kinds, Y, X):
           ph.optics(na_ill=0.4, tilt_x=-0.6, tilt_y=0.3)]
     banks = []
     for general in (False, True):
-        tf = torch.full((B.wo_tf_bytes(3, 5, Y, X, k),), 0x7F, dtype=torch.uint8, device=dev)
-        ws = torch.full((B.wo_aberrated_workspace_bytes(3, 5, Y, X, k),), 0x7F, dtype=torch.uint8, device=dev)
+        tf = torch.full((B.wo_tf_bytes(3, 3, Y, X, k),), 0x7F, dtype=torch.uint8, device=dev)
+        ws = torch.full((B.wo_aberrated_workspace_bytes(3, 3, Y, X, k),), 0x7F, dtype=torch.uint8, device=dev)
         if general:
-            B.wo_build_tf_aberrated(ol, [[0.0]] * 3, 3, 5, Y, X, k, tf, ws)
+            B.wo_build_tf_aberrated(ol, [[0.0]] * 3, 3, 3, Y, X, k, tf, ws)
         else:
-            B.wo_build_tf(ol, 3, 5, Y, X, k, tf, ws)
-        banks.append(B.tf_views(tf, 3, 5, Y, X, k)[0])
+            B.wo_build_tf(ol, 3, 3, Y, X, k, tf, ws)
+        banks.append(B.tf_views(tf, 3, 3, Y, X, k)[0])
     assert torch.equal(banks[0], banks[1])
+
+
+@pytest.mark.parametrize("mode", ["3d", "2d"])
+@pytest.mark.parametrize("Z", [8, 12, 16, 24, 32, 48, 64, 96, 128])
+def test_fusion_at_every_plane_count(env, Z, mode):
+    """Register columns (12 to 64, 128) and shared-memory ones, a last partial CTA, relative regulariser."""
+    B, torch, dev = env
+    n, C, Y, X = 2, 3, 6, 32
+    ol = [ph.optics(na_ill=0.15, tilt_x=0.5 * np.cos(a), tilt_y=0.5 * np.sin(a)) for a in range(n * C)]
+    tf, ws0 = B.alloc(n * C, Z, Y, X, "phase", dev)
+    B.wo_build_tf(ol, n * C, Z, Y, X, "phase", tf, ws0)
+    H = B.tf_views(tf, n * C, Z, Y, X, 1)[0].to(torch.complex128).reshape(n, C, Z, Y, X // 2 + 1)
+    d = noise(torch, dev, Z, n, C, Z, Y, X)
+    D = torch.fft.rfftn(d.double(), dim=(-3, -2, -1))
+    D[..., 0, 0, 0] = 0  # the default background is the channel's mean
+    ws = torch.full((B.wo_fused_workspace_bytes(C, n, Z, Y, X),), 0xFF, dtype=torch.uint8, device=dev)
+    two = mode == "2d"
+    out = torch.empty((n, Y, X) if two else (n, Z, Y, X), device=dev)
+    B.wo_reconstruct_fused(tf, C, d, None, 0.05, B.WO_ETA_RELATIVE, B.WO_MODE_2D if two else B.WO_MODE_3D, out, n, Z,
+                           Y, X, ws)
+    num, den = (H.conj() * D).sum(1), (H.abs() ** 2).sum(1)
+    if two:
+        num, den = num.sum(1), den.sum(1)
+    lam = 0.05 * den.amax(dim=tuple(range(1, den.dim())), keepdim=True)
+    want = torch.fft.irfftn(num / (den + lam), s=(Y, X) if two else (Z, Y, X), dim=(-2, -1) if two else (-3, -2, -1))
+    assert rel(torch, out, want) < 5e-6
