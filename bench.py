@@ -66,10 +66,10 @@ CPU_SAMPLE = (96, 256, 256)
 # capture), scaled by 4 to the 256 tiles of a launch of the bench's field
 # (the traffic grows with the tiles).
 NCU_TRAFFIC = {
-    ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "7cdb369169da44ec"},
-    ("field", "tf_psf_rows"): {"bytes": 4 * (584036096 + 423149568), "digest": "5f1f936b431924f0"},
-    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "5556489b6f389c1b"},
-    ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "5556489b6f389c1b"},
+    ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "eca89ebaa6186dda"},
+    ("field", "tf_psf_rows"): {"bytes": 4 * (584036096 + 423149568), "digest": "dea6d3be6c800244"},
+    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "4edc7bbde037b88b"},
+    ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "4edc7bbde037b88b"},
 }
 
 

@@ -206,4 +206,73 @@ struct Row512 {
   }
 };
 
+// 384 points on a half warp, 24 per lane (lane l owns p = l + 16 m): Stockham
+// passes of radix 24 (from registers), 8 and 2, with two exchanges through a
+// slice padded by one element per 24 (index p + p/24): the first pass's
+// writes (stride 25) and the runs of 16 of the others fall on distinct 8-byte
+// bank pairs but for one pair where a run crosses a pad.
+struct Row384 {
+  static constexpr int N = 384, E = 24, T = 16;
+  static constexpr int SLICE = N + N / 24;
+  static constexpr int TW = N + 192;  // w_384^m, then w_192^(r k) at [r * 24 + k]
+
+  static __device__ __forceinline__ int pad(int p) { return p + p / 24; }
+
+  static __device__ __forceinline__ void twiddles(float2* tw) {
+    make_twiddles<N>(tw);
+    for (int e = threadIdx.x; e < 192; e += blockDim.x) {
+      const int r = e / 24, k = e % 24;
+      float s, c;
+      sincospif(2.0f * (float)(r * k) / 192.0f, &s, &c);
+      tw[N + e] = make_float2(c, -s);
+    }
+  }
+
+  template <bool INV, int SC = 0>
+  static __device__ __forceinline__ void fft(float2 (&v)[E], const float2* tw, float2* S, int l) {
+    // pass 1 (sub-length 1, radix 24): butterfly l takes points l + 16 r
+    reg_stages<24, 1, INV, 16, SC>(v, tw);
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 24; ++r) S[25 * l + r] = v[r];
+    __syncwarp();
+    // pass 2 (sub-length 24, radix 8): butterflies j = l + 16 i, twiddles w_192^(r k), k = j mod 24
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int j = l + 16 * i, k = j % 24;
+      float2 u[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        u[r] = S[pad(j) + 50 * r];  // pad(j + 48 r)
+        if (r > 0) {
+          float2 w = tw[N + r * 24 + k];
+          if (INV) w.y = -w.y;
+          u[r] = cmul(u[r], w);
+        }
+      }
+      dft8<INV>(u);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[8 * i + r] = u[r];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int j = l + 16 * i, base = (j / 24) * 200 + j % 24;  // pad((j / 24) 192 + j mod 24)
+#pragma unroll
+      for (int r = 0; r < 8; ++r) S[base + 25 * r] = v[8 * i + r];
+    }
+    __syncwarp();
+    // pass 3 (sub-length 192, radix 2): butterflies j = l + 16 i, twiddle w_384^j
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      const int j = l + 16 * i, q = pad(j);
+      float2 w = tw[j];
+      if (INV) w.y = -w.y;
+      const float2 a = S[q], b = cmul(S[q + 200], w);  // pad(j + 192)
+      v[i] = cadd(a, b);
+      v[i + 12] = csub(a, b);
+    }
+  }
+};
+
 }  // namespace wo

@@ -398,6 +398,7 @@ cudaError_t launch_c2r_reg(const float2* in, float* out, long long nrows, float 
 
 }  // namespace
 
+// The lengths whose engine the schedule may choose (and the tile passes take).
 bool rows_reg_supported(int N) {
   return N == 32 || N == 48 || N == 64 || N == 96 || N == 128 || N == 192 || N == 256 || N == 512;
 }
@@ -411,6 +412,7 @@ cudaError_t rows_r2c_reg(int N, const float* in, float2* out, long long nrows, R
     case 128: return launch_r2c_reg<Row2<128, 16>>(in, out, nrows, bg, s);
     case 192: return launch_r2c_reg<Row2<192, 24>>(in, out, nrows, bg, s);
     case 256: return launch_r2c_reg<Row2<256, 16>>(in, out, nrows, bg, s);
+    case 384: return launch_r2c_reg<Row384>(in, out, nrows, bg, s);
     case 512: return launch_r2c_reg<Row512>(in, out, nrows, bg, s);
     default: return cudaErrorInvalidValue;
   }
@@ -496,6 +498,7 @@ cudaError_t rows_c2r_reg(int N, const float2* in, float* out, long long nrows, f
     case 128: return launch_c2r_reg<Row2<128, 16>>(in, out, nrows, scale, bg, s);
     case 192: return launch_c2r_reg<Row2<192, 24>>(in, out, nrows, scale, bg, s);
     case 256: return launch_c2r_reg<Row2<256, 16>>(in, out, nrows, scale, bg, s);
+    case 384: return launch_c2r_reg<Row384>(in, out, nrows, scale, bg, s);
     case 512: return launch_c2r_reg<Row512>(in, out, nrows, scale, bg, s);
     default: return cudaErrorInvalidValue;
   }

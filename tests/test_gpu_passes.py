@@ -35,9 +35,10 @@ def noise(torch, dev, seed, *shape):
 
 
 @pytest.mark.parametrize("Y", [2, 3, 6, 8, 12, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 2048])
-@pytest.mark.parametrize("X", [2, 96])
+@pytest.mark.parametrize("X", [2, 96, 768])
 def test_plane_spectra_at_every_column_length(env, Y, X):
-    """Columns of one to four stages, strips of one, 16 and a last odd column."""
+    """Columns of one to four stages, strips of one, 16 and a last odd column;
+    rows of 768 samples."""
     B, torch, dev = env
     d = noise(torch, dev, Y, 2, 3, Y, X)
     spec = torch.empty((2, 3, Y, X // 2 + 1), dtype=torch.complex64, device=dev)
