@@ -115,6 +115,51 @@ __device__ __forceinline__ bool outside_support(const float* stats, int y, int Y
   return fy * fy + fx * fx > r * r;
 }
 
+// The operator at one 3D frequency: the input volumes' values x to the output
+// volumes' values y (zero where the operator gives none), H the bank's slots
+// (zero past its last); dc: the reconstruction leaves this bin out.
+__device__ __forceinline__ void z_operator(const ZOp& op, const float2 (&H)[3], float2 x0v, float2 x1v, float2 x2v,
+                                           float lam_lf, float lam_fl, bool dc, float2& y0, float2& y1, float2& y2) {
+  const int L = op.lf_props;
+  const float2 zero = make_float2(0.f, 0.f);
+  if (op.op == 0) {  // forward: props in, channels out
+    if (L > 0) {
+      float2 d = cmul(H[0], x0v);
+      if (L > 1) d = cadd(d, cmul(H[1], x1v));
+      if (op.lf_chan == 0) y0 = d; else y1 = d;
+    }
+    if (op.has_fl) {
+      const float2 d = cmul(H[L], sel3(L, x0v, x1v, x2v));
+      if (op.fl_chan == 0) y0 = d; else y1 = d;
+    }
+  } else if (op.op == 1) {  // adjoint: channels in, props out
+    if (L > 0) {
+      const float2 d = sel3(op.lf_chan, x0v, x1v, x2v);
+      y0 = cmulc(H[0], d);
+      if (L > 1) y1 = cmulc(H[1], d);
+    }
+    if (op.has_fl) {
+      const float2 f = cmulc(H[L], sel3(op.fl_chan, x0v, x1v, x2v));
+      if (L == 0) y0 = f; else if (L == 1) y1 = f; else y2 = f;
+    }
+  } else {  // reconstruct
+    if (L > 0) {
+      const float2 d = dc ? zero : sel3(op.lf_chan, x0v, x1v, x2v);
+      float den = lam_lf + cabs2(H[0]);
+      if (L > 1) den += cabs2(H[1]);
+      const float inv = den > 0.f ? 1.0f / den : 0.f;  // zero TF and eta: minimum norm
+      y0 = cscale(cmulc(H[0], d), inv);
+      if (L > 1) y1 = cscale(cmulc(H[1], d), inv);
+    }
+    if (op.has_fl) {
+      const float2 d = dc ? zero : sel3(op.fl_chan, x0v, x1v, x2v);
+      const float den = lam_fl + cabs2(H[L]);
+      const float2 f = cscale(cmulc(H[L], d), den > 0.f ? 1.0f / den : 0.f);
+      if (L == 0) y0 = f; else if (L == 1) y1 = f; else y2 = f;
+    }
+  }
+}
+
 template <int N, int NI, int NO>
 __global__ void __launch_bounds__(ZGeom<N, (NI > NO ? NI : NO)>::NT, ZGeom<N, (NI > NO ? NI : NO)>::MINB)
     k_z_fused(const float2* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tf, ZOp op,
@@ -159,7 +204,6 @@ __global__ void __launch_bounds__(ZGeom<N, (NI > NO ? NI : NO)>::NT, ZGeom<N, (N
   const float* st = op.stats + (long long)tt * 8;
   const float lam_lf = op.eta_absolute ? op.eta_lf : op.eta_lf * st[0];
   const float lam_fl = op.eta_absolute ? op.eta_fl : op.eta_fl * st[2];
-  const int L = op.lf_props;
   const float2 zero = make_float2(0.f, 0.f);
   // a thread keeps one column b (NT is a multiple of B); columns outside the
   // support disk hold only the TFs' rounding noise: zero out
@@ -178,43 +222,7 @@ __global__ void __launch_bounds__(ZGeom<N, (NI > NO ? NI : NO)>::NT, ZGeom<N, (N
       float2 H[3];
 #pragma unroll
       for (int s = 0; s < 3; ++s) H[s] = (s < ntf) ? h[s * N * B] : zero;
-      if (op.op == 0) {  // forward: props in, channels out
-        if (L > 0) {
-          float2 d = cmul(H[0], x0v);
-          if (L > 1) d = cadd(d, cmul(H[1], x1v));
-          if (op.lf_chan == 0) y0 = d; else y1 = d;
-        }
-        if (op.has_fl) {
-          const float2 d = cmul(H[L], sel3(L, x0v, x1v, x2v));
-          if (op.fl_chan == 0) y0 = d; else y1 = d;
-        }
-      } else if (op.op == 1) {  // adjoint: channels in, props out
-        if (L > 0) {
-          const float2 d = sel3(op.lf_chan, x0v, x1v, x2v);
-          y0 = cmulc(H[0], d);
-          if (L > 1) y1 = cmulc(H[1], d);
-        }
-        if (op.has_fl) {
-          const float2 f = cmulc(H[L], sel3(op.fl_chan, x0v, x1v, x2v));
-          if (L == 0) y0 = f; else if (L == 1) y1 = f; else y2 = f;
-        }
-      } else {  // reconstruct
-        const bool dc = op.zero_dc && k == 0 && y == 0 && (x0 + b) == 0;
-        if (L > 0) {
-          const float2 d = dc ? zero : sel3(op.lf_chan, x0v, x1v, x2v);
-          float den = lam_lf + cabs2(H[0]);
-          if (L > 1) den += cabs2(H[1]);
-          const float inv = den > 0.f ? 1.0f / den : 0.f;  // zero TF and eta: minimum norm
-          y0 = cscale(cmulc(H[0], d), inv);
-          if (L > 1) y1 = cscale(cmulc(H[1], d), inv);
-        }
-        if (op.has_fl) {
-          const float2 d = dc ? zero : sel3(op.fl_chan, x0v, x1v, x2v);
-          const float den = lam_fl + cabs2(H[L]);
-          const float2 f = cscale(cmulc(H[L], d), den > 0.f ? 1.0f / den : 0.f);
-          if (L == 0) y0 = f; else if (L == 1) y1 = f; else y2 = f;
-        }
-      }
+      z_operator(op, H, x0v, x1v, x2v, lam_lf, lam_fl, op.zero_dc && k == 0 && y == 0 && (x0 + b) == 0, y0, y1, y2);
     }
     cell[0] = y0;
     if (NO > 1) cell[B] = y1;
@@ -223,6 +231,152 @@ __global__ void __launch_bounds__(ZGeom<N, (NI > NO ? NI : NO)>::NT, ZGeom<N, (N
   __syncthreads();
   fft_smem<N, NO * B, NT, true, 1>(buf, NV * B, 1, tw);
   store_zcols<N, NV, B, NT>(buf, out + (long long)t * NO * vol + col, NO, vol, zs, w);
+}
+
+// ------------------------------------------------- the z pass through registers
+// Radices of a length-N transform: stage i of the forward one.
+__host__ __device__ constexpr int z_stages(int N) { return N == 1 ? 0 : 1 + z_stages(N / radix_for(N)); }
+__host__ __device__ constexpr int z_radix(int N, int i) { return i == 0 ? radix_for(N) : z_radix(N / radix_for(N), i - 1); }
+
+template <int N, int NI, int NO>
+struct ZThruGeom {
+  static constexpr int S = z_stages(N), RL = z_radix(N, S - 1), ML = N / RL;
+  // columns per CTA: 64-byte runs or whole 128-byte lines, a last-stage butterfly a thread
+  static constexpr int B = ML >= 32 ? 8 : ML >= 8 ? 16 : 128 / ML;
+  static constexpr int NT = ML * B;
+  static constexpr int MINB = (RL == 8 ? 512 : 1024) / NT;  // eight points, volumes and TFs a thread: 128 registers
+  static constexpr int NV = NI > NO ? NI : NO;
+  static constexpr size_t SMEM = ((size_t)N + (S > 1 ? (size_t)NV * N * B : 0)) * sizeof(float2);
+};
+
+// Forward stages 0 .. S - 2 of NI volumes' columns (sequence v B + b) into buf.
+template <int N, int SB, int NT, int I, int NS, class In, class Out>
+__device__ __forceinline__ void z_forward(float2* buf, float2* tw, In in, Out out) {
+  if constexpr (I + 1 < z_stages(N)) {
+    constexpr int R = z_radix(N, I);
+    fft_stage_io<N, SB, NT, false, R, NS, I == 0, I == 0>(buf, tw, threadIdx.x, in, out);
+    z_forward<N, SB, NT, I + 1, NS * R>(buf, tw, in, out);
+  }
+}
+
+// Inverse stages 1 .. S - 1, the radices in reverse order, the last into out.
+template <int N, int SB, int NT, int I, int NS, class In, class Out>
+__device__ __forceinline__ void z_inverse(float2* buf, float2* tw, In in, Out out) {
+  if constexpr (I < z_stages(N)) {
+    constexpr int R = z_radix(N, z_stages(N) - 1 - I);
+    fft_stage_io<N, SB, NT, true, R, NS, false, false>(buf, tw, threadIdx.x, in, out);
+    z_inverse<N, SB, NT, I + 1, NS * R>(buf, tw, in, out);
+  }
+}
+
+// k_z_fused without the copies: the first forward stage loads from global
+// memory, the last one, the operator and the first inverse stage share a
+// thread's registers (the inverse takes the radices in reverse order, so its
+// first butterfly wants just the frequencies k0 + r N / R that the last
+// forward butterfly leaves), and the last inverse stage stores to global
+// memory.  A point passes through shared memory four times instead of
+// sixteen (three stages), the transfer functions not at all: their loads are
+// issued before the first stage.  The columns of a tile's planes are taken in
+// the order of memory (B of y Xh + x), so every line is whole where Y Xh is a
+// multiple of 16.  Phase and
+// fluorescence, 2 x 24x384x385: 89 -> 63 us; all kinds reconstructed from two
+// volumes, 96x512x257: 202 -> 175 us (16 columns a CTA there: 194 us).
+template <int N, int NI, int NO>
+__global__ void __launch_bounds__(ZThruGeom<N, NI, NO>::NT, ZThruGeom<N, NI, NO>::MINB)
+    k_z_thru(const float2* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tf, ZOp op, int Y,
+             int Xh) {
+  using G = ZThruGeom<N, NI, NO>;
+  constexpr int B = G::B, NT = G::NT, RL = G::RL, ML = G::ML, S = G::S;
+  extern __shared__ float2 sm[];
+  float2* tw = sm;
+  float2* buf = sm + N;
+  const int t = blockIdx.y, X = 2 * (Xh - 1);
+  const int zs = Y * Xh, c0 = blockIdx.x * B;  // (zs <= 2048 * 1025)
+  const long long vol = (long long)N * zs;
+  const int tt = op.tf_shared ? 0 : t;  // the tile whose TFs and statistics apply
+  const float* st = op.stats + (long long)tt * 8;
+  // the column that a sequence v B + b of this thread belongs to: b = tid % B
+  // in every stage (NT is a multiple of B, and so is the sequences' number)
+  const int b = threadIdx.x % B, c = c0 + b;
+  const bool live = c < zs;
+  const int y = c / Xh, x = c - y * Xh;
+  const bool inside = live && !outside_support(st, y, Y, x, X);
+#if defined(WO_CHECK) && WO_CHECK
+  {  // the strip's last elements in the input, output and TF volumes
+    const long long last = (long long)(N - 1) * zs + min(c0 + B, zs) - 1;
+    const long long nt = gridDim.y, ntt = op.tf_shared ? 1 : nt;
+    if (!WO_IN((long long)t * NI * vol + (NI - 1) * vol + last, nt * NI * vol, 6) ||
+        !WO_IN((long long)t * NO * vol + (NO - 1) * vol + last, nt * NO * vol, 6) ||
+        !WO_IN((long long)tt * op.n_tf * vol + (op.n_tf - 1) * vol + last, ntt * op.n_tf * vol, 6))
+      return;  // uniform across the CTA
+  }
+#endif
+  float2* dst = out + (long long)t * NO * vol + c;
+  const float2 zero = make_float2(0.f, 0.f);
+  if (!__syncthreads_or(inside)) {  // every TF is zero here, so is every operator's output
+    if (live) {
+      for (int v = 0; v < NO; ++v)
+        for (int n = threadIdx.x / B; n < N; n += NT / B) dst[v * vol + (long long)n * zs] = zero;
+    }
+    return;  // uniform across the CTA
+  }
+  const float2* src = in + (long long)t * NI * vol + c;
+  const float2* h = tf + (long long)tt * op.n_tf * vol + c;
+  const int k0 = threadIdx.x / B;  // this thread's last-stage butterfly: frequencies k0 + r ML
+  float2 H[RL][3];
+#pragma unroll
+  for (int r = 0; r < RL; ++r) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      H[r][q] = (inside && q < op.n_tf) ? __ldg(h + q * vol + (long long)(k0 + r * ML) * zs) : zero;
+  }
+  auto load = [&](int n, int s, int) { return inside ? __ldg(src + (s / B) * vol + (long long)n * zs) : zero; };
+  auto store = [&](int n, int s, float2 v) {
+    if (live) dst[(s / B) * vol + (long long)n * zs] = inside ? v : zero;
+  };
+  auto none = [](int, int, float2) {};
+  z_forward<N, NI * B, NT, 0, 1>(buf, tw, load, none);
+  float2 xv[3][RL];
+#pragma unroll
+  for (int v = 0; v < NI; ++v) {
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      const int n = k0 + r * ML;
+      if constexpr (S == 1) {
+        xv[v][r] = load(n, v * B, 0);
+      } else {
+        xv[v][r] = buf[n * (NI * B) + v * B + b];
+        if (r > 0) xv[v][r] = cmul(xv[v][r], tw[r * k0]);  // (k0 < NS = ML: twiddle w_N^(r k0))
+      }
+    }
+    dftR<RL, false>(xv[v]);
+  }
+  const float lam_lf = op.eta_absolute ? op.eta_lf : op.eta_lf * st[0];
+  const float lam_fl = op.eta_absolute ? op.eta_fl : op.eta_fl * st[2];
+#pragma unroll
+  for (int r = 0; r < RL; ++r) {
+    float2 y0 = zero, y1 = zero, y2 = zero;
+    if (inside)
+      z_operator(op, H[r], xv[0][r], NI > 1 ? xv[1][r] : zero, NI > 2 ? xv[2][r] : zero, lam_lf, lam_fl,
+                 op.zero_dc && c == 0 && k0 + r * ML == 0, y0, y1, y2);
+    xv[0][r] = y0;
+    if (NO > 1) xv[1][r] = y1;
+    if (NO > 2) xv[2][r] = y2;
+  }
+  if (S > 1) __syncthreads();  // the forward stages' reads of buf are done
+#pragma unroll
+  for (int v = 0; v < NO; ++v) {
+    dftR<RL, true>(xv[v]);
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      if constexpr (S == 1) store(r, v * B, xv[v][r]);
+      else buf[(k0 * RL + r) * (NO * B) + v * B + b] = xv[v][r];
+    }
+  }
+  if constexpr (S > 1) {
+    __syncthreads();
+    z_inverse<N, NO * B, NT, 1, RL>(buf, tw, load, store);
+  }
 }
 
 // 2D: out[t][p][y][x] = (sum_k H_k^H H_k + lam I)^-1 sum_k H_k^H D_k per mode.
@@ -342,6 +496,15 @@ template <int N, int NI, int NO>
 cudaError_t launch_z_fused(const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles, int Y, int Xh,
                            cudaStream_t s) {
   constexpr int NV = NI > NO ? NI : NO;
+  // one plane has no transform; past 192 the last stage's butterflies outnumber a CTA's threads
+  if constexpr (N > 1 && N <= 192) {
+    using G = ZThruGeom<N, NI, NO>;
+    const cudaError_t attr = allow_smem(k_z_thru<N, NI, NO>, G::SMEM);
+    if (attr != cudaSuccess) return attr;
+    dim3 grid((unsigned)((Y * Xh + G::B - 1) / G::B), (unsigned)n_tiles);
+    WO_LAUNCH("z_fused", s, (k_z_thru<N, NI, NO><<<grid, G::NT, G::SMEM, s>>>(in, out, tf, op, Y, Xh)));
+    return cudaGetLastError();
+  }
   using G = ZGeom<N, NV>;
   const cudaError_t attr = allow_smem(k_z_fused<N, NI, NO>, G::SMEM_TF);
   if (attr != cudaSuccess) return attr;
