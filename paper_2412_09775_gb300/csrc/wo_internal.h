@@ -102,6 +102,9 @@ cudaError_t z_fused(int Z, const float2* in, float2* out, const float2* tf, ZOp 
 bool z_reg_supported(int Z, const ZOp& op);
 cudaError_t z_fused_reg(int Z, const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles, int Y, int Xh,
                         cudaStream_t s);
+bool z_solve_reg_supported(int Z, const ZOp& op);
+cudaError_t z_solve_reg(int Z, const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles, int Y, int Xh,
+                        cudaStream_t s);
 // 2D reconstruction: FFT_z, per-transverse-frequency solve summed over k_z.
 // out: [tile][P][Y][Xh].
 cudaError_t z_solve2d(int Z, const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles,

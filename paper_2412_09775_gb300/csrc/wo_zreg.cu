@@ -117,6 +117,90 @@ cudaError_t launch_z_reg(const float2* in, float2* out, const float2* tf, ZOp op
   return cudaGetLastError();
 }
 
+// The 2D solve of the same systems (k_z_solve2d with one volume, one TF):
+//   F = sum_k conj(H_k) D~_k / (sum_k |H_k|^2 + eta)
+// per transverse frequency, D~ transformed along z in registers, the sums over
+// a column's lanes by shuffles.  The columns are taken in the order of memory
+// (CPC of y Xh + x); a CTA whose columns all lie outside the support reads
+// nothing.  The shared-memory kernel moved every column through a tile and 11
+// sums through shared memory: 36 x 24x256x256 96 -> 58 us.
+template <class P>
+__global__ void __launch_bounds__(ZRegGeom<P>::NT) k_z_solve_reg(const float2* __restrict__ in,
+                                                                float2* __restrict__ out,
+                                                                const float2* __restrict__ tf, ZOp op, int Y, int Xh) {
+  using G = ZRegGeom<P>;
+  constexpr int N = G::N, T = G::T, E = G::E, CPC = G::CPC;
+  extern __shared__ float2 sm[];
+  float2* tw = sm;
+  const int l = threadIdx.x % T, cl = threadIdx.x / T;
+  float2* S = sm + P::TW + cl * P::SLICE;
+  const int t = blockIdx.y, zs = Y * Xh, c = blockIdx.x * CPC + cl;
+  const long long vol = (long long)N * zs;
+  const int tt = op.tf_shared ? 0 : t;  // the tile whose TF and statistics apply
+  const float* st = op.stats + (long long)tt * 8;
+#if defined(WO_CHECK) && WO_CHECK
+  {  // the CTA's last elements in the input and TF volumes and in the 2D output
+    const long long end = min((int)(blockIdx.x + 1) * CPC, zs) - 1, last = (long long)(N - 1) * zs + end;
+    const long long nt = gridDim.y, ntt = op.tf_shared ? 1 : nt;
+    if (!WO_IN((long long)t * vol + last, nt * vol, 6) || !WO_IN((long long)tt * vol + last, ntt * vol, 6) ||
+        !WO_IN((long long)t * zs + end, nt * zs, 6))
+      return;  // uniform across the CTA
+  }
+#endif
+  const bool live = c < zs;
+  const int y = c / Xh, x = c - y * Xh;
+  const bool inside = live && !outside_support(st, y, Y, x, 2 * (Xh - 1));
+  float2* o = out + (long long)t * zs + c;
+  if (!__syncthreads_or(inside)) {
+    if (live && l == 0) *o = make_float2(0.f, 0.f);
+    return;  // uniform across the CTA
+  }
+  const float2* src = in + (long long)t * vol + c;
+  const float2* h = tf + (long long)tt * vol + c;
+  float2 v[E], H[E];
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const long long q = (long long)(l + T * m) * zs;
+    v[m] = inside ? __ldg(src + q) : make_float2(0.f, 0.f);
+    H[m] = inside ? __ldg(h + q) : make_float2(0.f, 0.f);
+  }
+  P::twiddles(tw);  // while the loads are in flight
+  __syncthreads();
+  P::template fft<false>(v, tw, S, l);
+  if (op.zero_dc && c == 0 && l == 0) v[0] = make_float2(0.f, 0.f);
+  float2 num = make_float2(0.f, 0.f);
+  float den = 0.f;
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    num = cadd(num, cmulc(H[m], v[m]));
+    den += cabs2(H[m]);
+  }
+#pragma unroll
+  for (int s = 1; s < T; s <<= 1) {
+    num.x += __shfl_xor_sync(0xffffffffu, num.x, s);
+    num.y += __shfl_xor_sync(0xffffffffu, num.y, s);
+    den += __shfl_xor_sync(0xffffffffu, den, s);
+  }
+  if (live && l == 0) {
+    // per-plane sums are 1/Z of the sums over k, so an absolute eta enters as Z eta
+    const bool lf = op.lf_props > 0;
+    const float eta = lf ? op.eta_lf : op.eta_fl;
+    const float q = den + (op.eta_absolute ? eta * (float)N : eta * st[lf ? 1 : 3]);
+    *o = cscale(num, q > 0.f ? 1.0f / q : 0.f);
+  }
+}
+
+template <class P>
+cudaError_t launch_z_solve_reg(const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles, int Y, int Xh,
+                               cudaStream_t s) {
+  using G = ZRegGeom<P>;
+  const cudaError_t attr = allow_smem(k_z_solve_reg<P>, G::SMEM);
+  if (attr != cudaSuccess) return attr;
+  dim3 grid((unsigned)((Y * Xh + G::CPC - 1) / G::CPC), (unsigned)n_tiles);
+  WO_LAUNCH("z_solve2d", s, (k_z_solve_reg<P><<<grid, G::NT, G::SMEM, s>>>(in, out, tf, op, Y, Xh)));
+  return cudaGetLastError();
+}
+
 // The TF build's z pass for one-kind banks (the same scheme): forward
 // transform along z of every TF column in place, and the per-tile maxima the
 // relative regulariser uses — max over (k, column) of |H|^2 and max over
@@ -214,6 +298,29 @@ cudaError_t tf_zpass_reg(const TfArgs& a, cudaStream_t s) {
     case 96: return launch_tf_zpass_reg<Row2<96, 24>>(a, s);
     case 128: return launch_tf_zpass_reg<Row2<128, 16>>(a, s);
     case 192: return launch_tf_zpass_reg<Row2<192, 24>>(a, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// One volume, one TF, and a plane count that divides among at most eight lanes.
+bool z_solve_reg_supported(int Z, const ZOp& op) {
+  if (op.n_in != 1 || op.n_tf != 1 || op.lf_props + op.has_fl != 1) return false;
+  return Z == 6 || Z == 8 || Z == 12 || Z == 16 || Z == 24 || Z == 32 || Z == 48 || Z == 64 || Z == 96 || Z == 128;
+}
+
+cudaError_t z_solve_reg(int Z, const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles, int Y, int Xh,
+                        cudaStream_t s) {
+  switch (Z) {
+    case 6: return launch_z_solve_reg<Row2<6, 6>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 8: return launch_z_solve_reg<Row2<8, 4>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 12: return launch_z_solve_reg<Row2<12, 6>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 16: return launch_z_solve_reg<Row2<16, 4>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 24: return launch_z_solve_reg<Row2<24, 12>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 32: return launch_z_solve_reg<Row2<32, 8>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 48: return launch_z_solve_reg<Row2<48, 12>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 64: return launch_z_solve_reg<Row2<64, 8>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 96: return launch_z_solve_reg<Row2<96, 24>>(in, out, tf, op, n_tiles, Y, Xh, s);
+    case 128: return launch_z_solve_reg<Row2<128, 16>>(in, out, tf, op, n_tiles, Y, Xh, s);
     default: return cudaErrorInvalidValue;
   }
 }
