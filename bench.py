@@ -68,8 +68,8 @@ CPU_SAMPLE = (96, 256, 256)
 NCU_TRAFFIC = {
     ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "eca89ebaa6186dda"},
     ("field", "tf_psf_rows"): {"bytes": 4 * (584036096 + 423149568), "digest": "dea6d3be6c800244"},
-    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "0e35e79d7ee4ff3c"},
-    ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "0e35e79d7ee4ff3c"},
+    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "19503de8fe03dbee"},
+    ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "19503de8fe03dbee"},
 }
 
 

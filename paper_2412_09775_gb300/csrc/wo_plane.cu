@@ -95,9 +95,12 @@ struct PlaneGeom {
   static constexpr int PLANE = Z * Y;
   // plane, y twiddles, z twiddles, one mbarrier per row
   static constexpr size_t SMEM = (size_t)(PLANE + Y + Z) * sizeof(float2) + (size_t)Z * sizeof(uint64_t);
-  // resident CTAs per SM by shared memory (228 KB per SM, 1 KB reserved per CTA, the static reduction array), at most 4
+  // resident CTAs per SM by shared memory (228 KB per SM, 1 KB reserved per CTA, the static reduction array), at
+  // most 4, or 8 of four warps where the transforms hold eight points a lane at most (64
+  // registers): 4096 stacks of 16x64x64, 33 planes each, 622 -> 601 us
   static constexpr int FIT = (int)((228 * 1024) / (SMEM + 1024 + 64));
-  static constexpr int MINB = FIT < 4 ? FIT : 4;
+  static constexpr int CAP = PY::E <= 8 && PZ::E <= 8 ? 1024 / NT : 4;
+  static constexpr int MINB = FIT < CAP ? FIT : CAP;
   static_assert(NT % 32 == 0 && Z % RPP == 0 && Y % CPP == 0, "whole passes of whole warps");
   static_assert(32 % PY::T == 0 && 32 % PZ::T == 0, "a row's or column's lanes sit in one warp");
   static_assert(Z % 2 == 0 && Y % 16 == 0 && Y > kRot, "row pairs; 16-byte rows; the odd-row rotation");
