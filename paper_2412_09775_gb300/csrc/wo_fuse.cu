@@ -29,8 +29,8 @@ struct FuseGeom {
 
 // Per tile: max over 3D frequencies of sum_c |H_c|^2 and max over transverse
 // frequencies of sum_k sum_c |H_c|^2 (the relative regulariser's scales in
-// 3D and 2D).  A CTA takes 32 (y, x) columns, eight of its warps' lanes each:
-// warp g sums the planes g, g + 8, ...  (One thread a column left the chip
+// 3D and 2D).  A CTA takes 32 (y, x) columns, one a lane of each of its eight
+// warps: warp g sums the planes g, g + 8, ...  (One thread a column left the chip
 // waiting on its 288 loads in turn: 4 tiles x 9 channels of 32x128x128 59.6 ->
 // 41 us.)
 __global__ void __launch_bounds__(256) k_fuse_stats(const float2* __restrict__ tf, int C, int Z, int Y, int Xh,

@@ -31,17 +31,19 @@ namespace wo {
 namespace {
 constexpr int kPsfThreads = 128;
 
-// even: the arm is stored for k_x >= 0 alone, column N - k stands for -k.
-template <class P>
+// EVEN: the arm is stored for k_x >= 0 alone, column N - k stands for -k.
+template <class P, bool EVEN = false>
 __device__ __forceinline__ void load_arm(float2 (&v)[P::E], const TfArgs& a, long long t, long long rem, int arm,
-                                         int kxm, int lane_t, bool even = false) {
+                                         int kxm, int lane_t) {
   constexpr int N = P::N, N1 = P::E, T = P::T;
   const float2* src = a.arms + ((t * a.n_arms + arm) * a.Z) * (long long)a.Y * N + rem * N;
+  const float2* pos = src + lane_t;
+  const float2* neg = EVEN ? src - lane_t : pos;
 #pragma unroll
   for (int m = 0; m < N1; ++m) {
     const int n = lane_t + T * m;
-    const int col = (2 * m >= N1 && even) ? N - n : n;
-    v[m] = (abs(fft_index(n, N)) <= kxm) ? __ldg(src + col) : make_float2(0.f, 0.f);
+    const float2* p = 2 * m < N1 ? pos + T * m : EVEN ? neg + (N - T * m) : neg + T * m;
+    v[m] = (abs(fft_index(n, N)) <= kxm) ? __ldg(p) : make_float2(0.f, 0.f);
   }
 }
 
@@ -60,7 +62,9 @@ __device__ __forceinline__ float2 mirror_value(const float2 (&v)[N1], int m, boo
 // derivative (arms A, B, A', B'); 2: plus the derivatives in tilt_x, tilt_y
 // and NA_ill under the smooth source (arms A_tx, A_ty, A_NA; their rows
 // 2K (Re conj(a_theta) b - (D_theta / D) Re g), D = sum S P^2).
-template <class P, int MODE>
+// BE: B and B' are stored for k_x >= 0 alone (TfArgs::b_even); a constant, so
+// that the loads' offsets are: 256 x 48x192x192 7.79 -> 7.47 ms.
+template <class P, int MODE, bool BE = false>
 __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4) k_psf_rows_reg(TfArgs a) {
   constexpr int N = P::N, N1 = P::E, T = P::T, RP = P::SLICE, RPC = kPsfThreads / T;
   __shared__ float2 tw[P::TW];
@@ -122,11 +126,11 @@ __global__ void __launch_bounds__(kPsfThreads, (P::E > 16 && MODE == 2) ? 2 : 4)
     if constexpr (DZ) {
       // w = 2K (Re conj(a) b + i (Re conj(a) b' + Re conj(a') b)), arms A, B, A', B'
       P::template fft<true>(va, tw, S, lt);
-      load_arm<P>(vb, a, t, rem, 3, kxm, lt, a.b_even != 0);
+      load_arm<P, BE>(vb, a, t, rem, 3, kxm, lt);
       P::template fft<true>(vb, tw, S, lt);
 #pragma unroll
       for (int m = 0; m < N1; ++m) w[m].y = va[m].x * vb[m].x + va[m].y * vb[m].y;
-      load_arm<P>(vb, a, t, rem, 1, kxm, lt, a.b_even != 0);
+      load_arm<P, BE>(vb, a, t, rem, 1, kxm, lt);
       P::template fft<true>(vb, tw, S, lt);
 #pragma unroll
       for (int m = 0; m < N1; ++m) w[m].x = va[m].x * vb[m].x + va[m].y * vb[m].y;
@@ -443,6 +447,10 @@ static cudaError_t launch_psf_reg(const TfArgs& a, cudaStream_t s) {
   constexpr int RPC = kPsfThreads / P::T;
   const long long rows = a.row_end - a.row_begin;
   const unsigned grid = (unsigned)((rows + RPC - 1) / RPC);
+  if (MODE > 0 && a.b_even) {
+    WO_LAUNCH("tf_psf_rows", s, (k_psf_rows_reg<P, MODE, (MODE > 0)><<<grid, kPsfThreads, 0, s>>>(a)));
+    return cudaGetLastError();
+  }
   WO_LAUNCH("tf_psf_rows", s, (k_psf_rows_reg<P, MODE><<<grid, kPsfThreads, 0, s>>>(a)));
   return cudaGetLastError();
 }
