@@ -434,28 +434,13 @@ __global__ void __launch_bounds__(kMmaThreads) k_conv_bwd_data_mma(const float* 
   float acc[NT][4];
 #pragma unroll
   for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
-  // the input ReLU's values at this thread's outputs, loaded now so that their
-  // latency hides under the stages (for the narrower layers, where the
-  // registers allow)
   const int g = lane >> 2, t = lane & 3;
-  constexpr bool kEarly = NT <= 8;
-  float xm[kEarly ? 4 : 1][kEarly ? NT : 1];
   // the input pixel of this thread's output rows (-1 past the class grid)
   auto out_pixel = [&](int q4) -> int {
     const int r = r0 + warp * 16 + g + (q4 >= 2 ? 8 : 0);
     const int i = r / W2, j = r - (r / W2) * W2;
     return r < NCLS ? (2 * i + ph) * H + 2 * j + pw : -1;
   };
-  if constexpr (kEarly) {
-    int xidx[4];
-#pragma unroll
-    for (int q4 = 0; q4 < 4; ++q4) xidx[q4] = out_pixel(q4);
-#pragma unroll
-    for (int q4 = 0; q4 < 4; ++q4)
-#pragma unroll
-      for (int n = 0; n < NT; ++n)
-        xm[q4][n] = xidx[q4] >= 0 ? __ldg(xin + ((long long)b * CI + n * 8 + 2 * t + (q4 & 1)) * H * H + xidx[q4]) : 0.f;
-  }
   load(0);
   store(0);
   __syncthreads();
@@ -490,11 +475,149 @@ __global__ void __launch_bounds__(kMmaThreads) k_conv_bwd_data_mma(const float* 
     for (int n = 0; n < NT; ++n) {
       const int ci = n * 8 + 2 * t + (q4 & 1);
       const long long idx = ((long long)b * CI + ci) * H * H + pix;
-      float xv;
-      if constexpr (kEarly) xv = xm[q4][n];
-      else xv = __ldg(xin + idx);
-      gx[idx] = xv > 0.f ? acc[n][q4] : 0.f;
+      gx[idx] = __ldg(xin + idx) > 0.f ? acc[n][q4] : 0.f;
     }
+  }
+}
+
+// The same for two classes of one row parity at once (pw = 0 and 1: the input
+// pixels (2 i + ph, 2 j) and (2 i + ph, 2 j + 1) of 64 pairs (i, j)).  One
+// class alone reads its masks and writes its gradients four bytes in eight, so
+// every sector of gx and xin crosses L2 twice; a pair moves whole 64-byte runs.
+// The window of gy at column j serves both classes (kw = 1 for pw = 0, kw = 2
+// for pw = 1), so three taps take two stagings and splits.  Every sum keeps its
+// order (kh, then kw = 0 before 2, then the channel chunks) and its bits.  For
+// CI <= 64, where the two classes' sums fit the registers.
+// 256 samples: 32 channels of 64 x 64 181 -> 144 us, 64 of 32 x 32 94 ->
+// 79 us.
+template <int CI, int CO, int H, int S>
+__global__ void __launch_bounds__(kMmaThreads) k_conv_bwd_data_pair(const float* __restrict__ gy,
+                                                                    const __nv_bfloat16* __restrict__ wtb,
+                                                                    const float* __restrict__ xin,
+                                                                    float* __restrict__ gx) {
+  constexpr int HO = H / 2, W2 = H / 2, NPAIR = W2 * W2, BPC = (NPAIR + 63) / 64, NT = CI / 8, P = kPitch32;
+  constexpr int BV = CI * 4 / kMmaThreads;  // 16-byte weight copies per thread, stage and tap
+  static_assert(S == 2 && H % 2 == 0, "the data gradient by parity classes is for stride 2");
+  static_assert(CI % 16 == 0 && CI <= 64 && CO % 32 == 0 && (CI * 4) % kMmaThreads == 0,
+                "channel counts of the paired data gradient");
+  __shared__ __align__(16) __nv_bfloat16 ahi[2][64 * P], alo[2][64 * P], bs[2][2][CI * P];
+  const int b = blockIdx.y, ph = blockIdx.x / BPC, r0 = (blockIdx.x - ph * BPC) * 64;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const StageLane sl;
+  int ci_[2], cj_[2];
+  bool rv[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int r = r0 + (2 * warp + h) * 8 + sl.m_lo;
+    rv[h] = r < NPAIR;
+    ci_[h] = r / W2;
+    cj_[h] = r - (r / W2) * W2;
+  }
+  const float* gb = gy + (long long)b * CO * HO * HO;
+  // stages (kernel row, dw = 1 then 0, 32-channel chunk); dw = 1 has one tap, dw = 0 two
+  constexpr int NCH = CO / 32;
+  const int nstage = (1 + ph) * 2 * NCH;
+  float av[2][4][2];  // [pixel][pair group][channel of the pair]
+  uint4 bv[2][BV];
+  auto load = [&](int st) {
+    const int c0 = (st % NCH) * 32, dw = 1 - (st / NCH) % 2, kh = ph ? 2 * (st / (2 * NCH)) : 1;
+    const int dh = (ph + 1 - kh) >> 1;  // output row i + dh, column j + dw
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int oh = ci_[h] + dh, ow = cj_[h] + dw;
+      const bool ok = rv[h] && oh < HO && ow < HO;
+      const float* src = gb + ((long long)(c0 + 2 * sl.p_lo) * HO + (ok ? oh : 0)) * HO + (ok ? ow : 0);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) av[h][q][c] = ok ? __ldg(src + (long long)(8 * q + c) * HO * HO) : 0.f;
+    }
+#pragma unroll
+    for (int pw = 0; pw < 2; ++pw) {  // pw = 0: kw = 1 (dw = 0 alone); pw = 1: kw = 0 (dw = 1) or 2
+      if (pw == 0 && dw == 1) continue;
+      const int kw = pw == 0 ? 1 : 2 - 2 * dw;
+      const uint4* wsrc = reinterpret_cast<const uint4*>(wtb + (long long)(kh * 3 + kw) * CI * CO + c0);
+#pragma unroll
+      for (int j = 0; j < BV; ++j) {
+        const int e = threadIdx.x + j * kMmaThreads, ci = e >> 2, q = e & 3;
+        bv[pw][j] = __ldg(wsrc + ci * (CO / 8) + q);
+      }
+    }
+  };
+  auto store = [&](int st, int buf) {
+    const int dw = 1 - (st / NCH) % 2;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int m = (2 * warp + h) * 8 + sl.m_lo;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float v0 = av[h][q][0], v1 = av[h][q][1];
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
+        const __nv_bfloat16 l0 = __float2bfloat16_rn(v0 - __bfloat162float(h0));
+        const __nv_bfloat16 l1 = __float2bfloat16_rn(v1 - __bfloat162float(h1));
+        const int o = m * P + 2 * (sl.p_lo + 4 * q);
+        *reinterpret_cast<__nv_bfloat162*>(&ahi[buf][o]) = __halves2bfloat162(h0, h1);
+        *reinterpret_cast<__nv_bfloat162*>(&alo[buf][o]) = __halves2bfloat162(l0, l1);
+      }
+    }
+#pragma unroll
+    for (int pw = 0; pw < 2; ++pw) {
+      if (pw == 0 && dw == 1) continue;
+#pragma unroll
+      for (int j = 0; j < BV; ++j) {
+        const int e = threadIdx.x + j * kMmaThreads, ci = e >> 2, q = e & 3;
+        *reinterpret_cast<uint4*>(&bs[buf][pw][ci * P + 8 * q]) = bv[pw][j];
+      }
+    }
+  };
+  float acc[2][NT][4];
+#pragma unroll
+  for (int pw = 0; pw < 2; ++pw)
+#pragma unroll
+    for (int n = 0; n < NT; ++n) acc[pw][n][0] = acc[pw][n][1] = acc[pw][n][2] = acc[pw][n][3] = 0.f;
+  load(0);
+  store(0, 0);
+  __syncthreads();
+  for (int st = 0; st < nstage; ++st) {
+    const int buf = st & 1, dw = 1 - (st / NCH) % 2;
+    if (st + 1 < nstage) load(st + 1);  // in flight during this stage's products
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      uint32_t fh[4], fl[4];
+      frag_a<P>(fh, ahi[buf] + warp * 16 * P + ks * 16, lane);
+      frag_a<P>(fl, alo[buf] + warp * 16 * P + ks * 16, lane);
+#pragma unroll
+      for (int pw = 0; pw < 2; ++pw) {
+        if (pw == 0 && dw == 1) continue;  // uniform
+#pragma unroll
+        for (int n = 0; n < NT; n += 2) {
+          uint32_t bb[4];
+          frag_b2<P>(bb, bs[buf][pw] + n * 8 * P + ks * 16, lane);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            mma16816(acc[pw][n + h], fl, bb[2 * h], bb[2 * h + 1]);
+            mma16816(acc[pw][n + h], fh, bb[2 * h], bb[2 * h + 1]);
+          }
+        }
+      }
+    }
+    if (st + 1 < nstage) store(st + 1, buf ^ 1);  // the other buffer was last read before the previous barrier
+    __syncthreads();
+  }
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int q4 = 0; q4 < 4; ++q4) {
+    const int r = r0 + warp * 16 + g + (q4 >= 2 ? 8 : 0);
+    if (r >= NPAIR) continue;
+    const int i = r / W2, j = r - (r / W2) * W2;
+    const long long base = ((long long)b * CI + 2 * t + (q4 & 1)) * H * H + (2 * i + ph) * H + 2 * j;
+    float2 xm[NT];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) xm[n] = __ldg(reinterpret_cast<const float2*>(xin + base + (long long)n * 8 * H * H));
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+      *reinterpret_cast<float2*>(gx + base + (long long)n * 8 * H * H) =
+          make_float2(xm[n].x > 0.f ? acc[0][n][q4] : 0.f, xm[n].y > 0.f ? acc[1][n][q4] : 0.f);
   }
 }
 
@@ -909,10 +1032,16 @@ cudaError_t bwd_layer(const float* gy, const float* xin, const __nv_bfloat16* wt
   e = cudaGetLastError();
   if (e != cudaSuccess || gx == nullptr) return e;
   if constexpr (CI % 8 == 0 && S == 2) {
-    dim3 gd((unsigned)(4 * ((H / 2 * (H / 2) + 63) / 64)), (unsigned)B);
+    constexpr unsigned kBlocks = (H / 2 * (H / 2) + 63) / 64;
     const char* dname = kDgName[layer_of<CI, CO, H, S>()];
-    WO_LAUNCH(dname, s, (k_conv_bwd_data_mma<CI, CO, H, S><<<gd, kMmaThreads, 0, s>>>(
-                            gy, wt + kConvTotal + conv_off(layer_of<CI, CO, H, S>()), xin, gx)));
+    const __nv_bfloat16* wb = wt + kConvTotal + conv_off(layer_of<CI, CO, H, S>());
+    if constexpr (CI <= 64) {
+      dim3 gd(2 * kBlocks, (unsigned)B);
+      WO_LAUNCH(dname, s, (k_conv_bwd_data_pair<CI, CO, H, S><<<gd, kMmaThreads, 0, s>>>(gy, wb, xin, gx)));
+    } else {
+      dim3 gd(4 * kBlocks, (unsigned)B);
+      WO_LAUNCH(dname, s, (k_conv_bwd_data_mma<CI, CO, H, S><<<gd, kMmaThreads, 0, s>>>(gy, wb, xin, gx)));
+    }
     return cudaGetLastError();
   }
   return cudaErrorInvalidValue;
