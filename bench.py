@@ -66,7 +66,7 @@ CPU_SAMPLE = (96, 256, 256)
 # capture), scaled by 4 to the 256 tiles of a launch of the bench's field
 # (the traffic grows with the tiles).
 NCU_TRAFFIC = {
-    ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "eca89ebaa6186dda"},
+    ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "c97e45a2f4971b23"},
     ("field", "tf_psf_rows"): {"bytes": 4 * (584036096 + 423149568), "digest": "4b80f0aa1abf3e4d"},
     ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "19503de8fe03dbee"},
     ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "19503de8fe03dbee"},

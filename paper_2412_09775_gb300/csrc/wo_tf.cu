@@ -672,6 +672,97 @@ __global__ void __launch_bounds__(ZGeom<N, NK>::NT, ZGeom<N, NK>::MINB) k_tf_zpa
   }
 }
 
+// The z pass by the scheme of k_z_thru (wo_zops.cuh): the first stage loads
+// from global memory, the last one keeps every kind's values of its
+// frequencies in registers, forms the maxima and stores.  The columns of a
+// tile in the order of memory; those with k_x >= x_cols are left as they are.
+// Three kinds, 96x512x257: 149 -> ZTHRU_US us.
+template <int N, int NK>
+__global__ void __launch_bounds__(ZThruGeom<N, NK, NK>::NT, ZThruGeom<N, NK, NK>::MINB) k_tf_zthru(TfArgs a) {
+  using G = ZThruGeom<N, NK, NK>;
+  constexpr int B = G::B, NT = G::NT, RL = G::RL, ML = G::ML, S = G::S;
+  extern __shared__ float2 sm[];
+  float2* tw = sm;
+  float2* buf = sm + N;
+  float* red = reinterpret_cast<float*>(sm + G::SMEM / sizeof(float2));  // [2][NT]
+  const int Xh = a.X / 2 + 1, zs = a.Y * Xh;
+  const int t = blockIdx.y, b = threadIdx.x % B, k0 = threadIdx.x / B, c = blockIdx.x * B + b;
+  const bool live = c < zs && c % Xh < a.x_cols;
+  const long long vol = (long long)N * zs;
+#if defined(WO_CHECK) && WO_CHECK
+  if (!WO_IN(((long long)t * NK + NK - 1) * vol + (long long)(N - 1) * zs + min((int)(blockIdx.x + 1) * B, zs) - 1,
+             (long long)gridDim.y * NK * vol, 6))
+    return;  // uniform across the CTA
+#endif
+  float2* base = a.tf + (long long)t * NK * vol + c;
+  const float2 zero = make_float2(0.f, 0.f);
+  auto load = [&](int n, int s, int) { return live ? base[(s / B) * vol + (long long)n * zs] : zero; };
+  z_forward<N, NK * B, NT, 0, 1>(buf, tw, load, [](int, int, float2) {});
+  const int L = a.lf_props;
+  float lf[RL], fl[RL];
+#pragma unroll
+  for (int r = 0; r < RL; ++r) lf[r] = fl[r] = 0.f;
+#pragma unroll
+  for (int v = 0; v < NK; ++v) {
+    float2 w[RL];
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      const int n = k0 + r * ML;
+      if constexpr (S == 1) {
+        w[r] = load(n, v * B, 0);
+      } else {
+        w[r] = buf[n * (NK * B) + v * B + b];
+        if (r > 0) w[r] = cmul(w[r], tw[r * k0]);
+      }
+    }
+    dftR<RL, false>(w);
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      if (live) base[v * vol + (long long)(k0 + r * ML) * zs] = w[r];
+      const float q = cabs2(w[r]);
+      if (v < L) lf[r] += q;
+      else if (v == L && a.want_fl) fl[r] += q;  // (a derivative slot counts in neither)
+    }
+  }
+  float m3_lf = 0.f, m3_fl = 0.f, col_lf = 0.f, col_fl = 0.f;
+#pragma unroll
+  for (int r = 0; r < RL; ++r) {
+    m3_lf = fmaxf(m3_lf, lf[r]);
+    m3_fl = fmaxf(m3_fl, fl[r]);
+    col_lf += lf[r];
+    col_fl += fl[r];
+  }
+  red[threadIdx.x] = col_lf;
+  red[NT + threadIdx.x] = col_fl;
+  __syncthreads();
+  float m2_lf = 0.f, m2_fl = 0.f;
+  if (k0 == 0) {
+    for (int q = 0; q < ML; ++q) {
+      m2_lf += red[q * B + b];
+      m2_fl += red[NT + q * B + b];
+    }
+  }
+  // maxima (values are >= 0, so integer order equals float order): over the
+  // warps, then one atomic per statistic and CTA
+  float m[4] = {m3_lf, m2_lf, m3_fl, m2_fl};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m[q] = fmaxf(m[q], __shfl_xor_sync(0xffffffffu, m[q], off));
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) red[4 * (threadIdx.x / 32) + q] = m[q];
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    float mx = 0.f;
+    for (int q = 0; q < NT / 32; ++q) mx = fmaxf(mx, red[4 * q + threadIdx.x]);
+    if (mx > 0.f) atomicMax(reinterpret_cast<int*>(a.stats + (long long)t * 8) + threadIdx.x, __float_as_int(mx));
+  }
+}
+
 cudaError_t tf_pupil_record(const TfArgs& a, cudaStream_t s) {
   const int kRecRows = record_rows(a.Y, a.n_tiles);
   dim3 grid((unsigned)((a.Y + kRecRows - 1) / kRecRows), (unsigned)a.n_tiles);
@@ -759,6 +850,16 @@ cudaError_t tf_psf_rows(const TfArgs& a, cudaStream_t s) {
 
 template <int N, int NK>
 static cudaError_t launch_zpass(const TfArgs& a, cudaStream_t s) {
+  if constexpr (N > 1 && N <= 192) {  // (the lengths of k_z_thru)
+    using G = ZThruGeom<N, NK, NK>;
+    constexpr size_t smem = G::SMEM + (size_t)2 * G::NT * sizeof(float);
+    const cudaError_t attr = allow_smem(k_tf_zthru<N, NK>, smem);
+    if (attr != cudaSuccess) return attr;
+    if (a.x_cols <= 0) return cudaSuccess;
+    dim3 grid((unsigned)((a.Y * (a.X / 2 + 1) + G::B - 1) / G::B), (unsigned)a.n_tiles);
+    WO_LAUNCH("tf_zpass", s, (k_tf_zthru<N, NK><<<grid, G::NT, smem, s>>>(a)));
+    return cudaGetLastError();
+  }
   using G = ZGeom<N, NK>;
   const size_t smem = G::SMEM + (size_t)G::NT * 2 * sizeof(float);
   const cudaError_t attr = allow_smem(k_tf_zpass<N, NK>, smem);
