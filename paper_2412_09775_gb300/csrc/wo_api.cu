@@ -604,7 +604,7 @@ static wo_status run_op(int op, const void* d_tf, unsigned kinds, const float* d
     WO_TRY(rows_r2c_field(H, *field, specA, in_rows, bg_in, cs));
     WO_TRY(cols_c2c(Y, false, specA, Xh, (long long)Y * Xh, Xh, in_rows / Y, cs, "y_fwd"));
   } else {
-    WO_TRY(plane_xy_fwd(X, Y, d_in, specA, in_rows / Y, bg_in, cs));
+    WO_TRY(plane_xy_fwd(X, Y, d_in, specA, in_rows / Y, bg_in, cs, xy_engine_for(X, Y, in_rows / Y)));
   }
   if (op == 2 && mode == WO_MODE_2D) {
     WO_TRY(z_solve2d(Z, specA, specB, tf, zo, n_tiles, Y, Xh, cs));
@@ -618,7 +618,8 @@ static wo_status run_op(int op, const void* d_tf, unsigned kinds, const float* d
       f2.Z = 1;
       WO_TRY(rows_c2r_blend(H, specB, f2, scale, cs));
     } else {
-      WO_TRY(plane_xy_inv(X, Y, specB, d_out, (long long)n_tiles * s.P, scale, none, cs));
+      const long long planes = (long long)n_tiles * s.P;
+      WO_TRY(plane_xy_inv(X, Y, specB, d_out, planes, scale, none, cs, xy_engine_for(X, Y, planes)));
     }
     return WO_OK;
   }
@@ -628,7 +629,8 @@ static wo_status run_op(int op, const void* d_tf, unsigned kinds, const float* d
     WO_TRY(cols_c2c(Y, true, specB, Xh, (long long)Y * Xh, Xh, (long long)n_tiles * n_out * Z, cs, "y_inv"));
     WO_TRY(rows_c2r_blend(H, specB, *fout, scale, cs));
   } else {
-    WO_TRY(plane_xy_inv(X, Y, specB, d_out, (long long)n_tiles * n_out * Z, scale, bg_out, cs));
+    const long long planes = (long long)n_tiles * n_out * Z;
+    WO_TRY(plane_xy_inv(X, Y, specB, d_out, planes, scale, bg_out, cs, xy_engine_for(X, Y, planes)));
   }
   return WO_OK;
 }

@@ -225,13 +225,24 @@ int cols_engine(int n);  // WO_ENGINE_SMEM or WO_ENGINE_HYBRID
 // The x and y transforms of a plane in one kernel per direction (wo_xy.cu),
 // and the helpers that pick it or the two passes by the schedule table.
 bool xy_supported(int X, int Y);
-int xy_engine(int X, int Y);  // WO_ENGINE_HYBRID: the fused kernels
+int xy_engine(int X, int Y);
+int xy_engine_for(int X, int Y, long long planes);  // WO_ENGINE_HYBRID: the fused kernels
 cudaError_t xy_fwd(int X, int Y, const float* in, float2* out, long long nplanes, RowBg bg, cudaStream_t s);
 cudaError_t xy_inv(int X, int Y, const float2* in, float* out, long long nplanes, float scale, RowBg bg,
                    cudaStream_t s);
-cudaError_t plane_xy_fwd(int X, int Y, const float* in, float2* out, long long nplanes, RowBg bg, cudaStream_t s);
+// `engine`: WO_ENGINE_HYBRID for the fused kernels.
+cudaError_t plane_xy_fwd(int X, int Y, const float* in, float2* out, long long nplanes, RowBg bg, cudaStream_t s,
+                         int engine);
 cudaError_t plane_xy_inv(int X, int Y, float2* in, float* out, long long nplanes, float scale, RowBg bg,
-                         cudaStream_t s);
+                         cudaStream_t s, int engine);
+inline cudaError_t plane_xy_fwd(int X, int Y, const float* in, float2* out, long long nplanes, RowBg bg,
+                                cudaStream_t s) {
+  return plane_xy_fwd(X, Y, in, out, nplanes, bg, s, xy_engine(X, Y));
+}
+inline cudaError_t plane_xy_inv(int X, int Y, float2* in, float* out, long long nplanes, float scale, RowBg bg,
+                                cudaStream_t s) {
+  return plane_xy_inv(X, Y, in, out, nplanes, scale, bg, s, xy_engine(X, Y));
+}
 int rows_engine(int n);  // engine of the x passes for n complex points (wo_rowsreg.cu: HYBRID)
 bool rows_reg_supported(int N);
 cudaError_t rows_r2c_reg(int N, const float* in, float2* out, long long nrows, RowBg bg, cudaStream_t s);

@@ -25,6 +25,7 @@ std::atomic<int> g_cols_engine[kMaxLen + 1];  // 0: default
 std::atomic<int> g_rows_engine[kMaxLen + 1];  // 0: default
 std::atomic<int> g_recon_engine[kMaxLen + 1];  // 0: default, keyed by Y
 std::atomic<int> g_xy_engine[kMaxLen + 1];     // 0: default, keyed by Y (X == Y)
+constexpr long long kXyFewPlanes = 768;
 }  // namespace
 
 int xy_engine(int X, int Y) {
@@ -38,6 +39,20 @@ int xy_engine(int X, int Y) {
   // 614 us per 64 tiles under ncu, 8 warps per SM); the autotuner keeps
   // them where they measure faster
   return WO_ENGINE_SMEM;
+}
+
+// The engine of an operator's xy passes over `planes` planes.  By default few
+// planes of 64 x 64 take the fused kernels: the launches are what such a call
+// waits for, and two of five fall away (16 to 64 planes 21 -> 17 us a
+// reconstruction, 256 planes 31.9 -> 25.2, 768 planes 47.4 -> 45.6).  Planes of
+// 128 x 128 and 192 x 192 lose even alone (21 -> 30 and 30 -> 47 us: one CTA a
+// plane).
+int xy_engine_for(int X, int Y, long long planes) {
+  if (!xy_supported(X, Y)) return WO_ENGINE_SMEM;
+  const int e = g_xy_engine[Y].load(std::memory_order_relaxed);
+  if (e != WO_ENGINE_SMEM && e != WO_ENGINE_HYBRID && X == 64 && Y == 64 && planes <= kXyFewPlanes)
+    return WO_ENGINE_HYBRID;
+  return xy_engine(X, Y);
 }
 
 int recon_engine(int Z, int Y, int X) {

@@ -282,10 +282,11 @@ cudaError_t xy_inv(int X, int Y, const float2* in, float* out, long long nplanes
   return xy_dispatch(true, X, Y, in, out, nplanes, scale, bg, s);
 }
 
-// The x and y transforms of nplanes planes: the fused kernel where the
-// schedule table says so, else the row pass and the column pass.
-cudaError_t plane_xy_fwd(int X, int Y, const float* in, float2* out, long long nplanes, RowBg bg, cudaStream_t s) {
-  if (xy_engine(X, Y) == WO_ENGINE_HYBRID) return xy_fwd(X, Y, in, out, nplanes, bg, s);
+// The x and y transforms of nplanes planes: the fused kernel or the row pass
+// and the column pass.
+cudaError_t plane_xy_fwd(int X, int Y, const float* in, float2* out, long long nplanes, RowBg bg, cudaStream_t s,
+                         int engine) {
+  if (engine == WO_ENGINE_HYBRID) return xy_fwd(X, Y, in, out, nplanes, bg, s);
   const int Xh = X / 2 + 1;
   const cudaError_t e = rows_r2c(X / 2, in, out, nplanes * Y, bg, s);
   if (e != cudaSuccess) return e;
@@ -294,8 +295,8 @@ cudaError_t plane_xy_fwd(int X, int Y, const float* in, float2* out, long long n
 
 // The inverse; the separate passes work in place on `in`.
 cudaError_t plane_xy_inv(int X, int Y, float2* in, float* out, long long nplanes, float scale, RowBg bg,
-                         cudaStream_t s) {
-  if (xy_engine(X, Y) == WO_ENGINE_HYBRID) return xy_inv(X, Y, in, out, nplanes, scale, bg, s);
+                         cudaStream_t s, int engine) {
+  if (engine == WO_ENGINE_HYBRID) return xy_inv(X, Y, in, out, nplanes, scale, bg, s);
   const int Xh = X / 2 + 1;
   const cudaError_t e = cols_c2c(Y, true, in, Xh, (long long)Y * Xh, Xh, nplanes, s, "y_inv");
   if (e != cudaSuccess) return e;
