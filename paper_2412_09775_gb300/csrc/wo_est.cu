@@ -61,17 +61,17 @@ __device__ __forceinline__ int freq_idx(int i, int n) { return (i < (n + 1) / 2)
 // power until k_feat_norm.
 //
 // Shared-memory float atomics bounded the former kernel (four a point, and
-// the neighbours of a ring meet in one bin).  Here two lanes of a warp share
-// 64 bins of {P, den, sx, sy} and add to them in turn (16 KB a warp; a slot
+// the neighbours of a ring meet in one bin).  Here four lanes of a warp share
+// 64 bins of {P, den, sx, sy} and add to them in turn (8 KB a warp; a slot
 // keeps its own banks whatever the bin), so a point costs one 16-byte load and
 // store and no atomic; the slots are summed at the end, in a fixed order.  The
 // rows y and Y - y of a plane share their frequencies' geometry and bin and
 // are added together.  Four warps take four rows r of one tile: the geometry
 // of 128 points at a time is formed once for them, and a warp's next plane is
 // its neighbour's plane (L1 hits).  Four points of a lane have their loads in
-// flight at once.  256 x 48x128x128: 1374 -> 616 us (one warp a CTA with a
-// slot a lane, the geometry formed by every warp: about 945 us).
-constexpr int kFeatRows = 4, kFeatPts = 32 * kFeatRows, kFeatSlots = 16;
+// flight at once.  256 x 48x128x128: 1374 -> 472 us (two lanes a slot, half the
+// warps an SM: 616; a slot a lane, the geometry formed by every warp: 945).
+constexpr int kFeatRows = 4, kFeatPts = 32 * kFeatRows, kFeatSlots = 8;
 
 __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict__ spec,
                                                        const wo_optics* __restrict__ optics, int Z, int Y, int X,
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
   float4* geo = sm4;                                                      // [2][128]: ux, uy, w, bin (-1: none)
   int2* off = reinterpret_cast<int2*>(geo + 2 * kFeatPts);                // [2][128]: the points at y and Y - y (-1: none)
   const int wi = threadIdx.x / 32, lane = threadIdx.x & 31;
-  float4* bins = reinterpret_cast<float4*>(off + 2 * kFeatPts) + wi * kSide * kFeatSlots;  // [64][16]
+  float4* bins = reinterpret_cast<float4*>(off + 2 * kFeatPts) + wi * kSide * kFeatSlots;  // [64][8]
   const int r = blockIdx.x * kFeatRows + wi, t = blockIdx.y;
   const int Xh = X / 2 + 1;
   const double pixel = optics[t].pixel_um, cut = 2.0 * optics[t].na_det / optics[t].lambda_um;
@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
         v.w = w * (ci - cm) * g[i].y;
       }
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {  // the slot's two lanes in turn
-        if (b >= 0 && lane / kFeatSlots == half) {
+      for (int turn = 0; turn < 32 / kFeatSlots; ++turn) {  // a slot's lanes in turn
+        if (b >= 0 && lane / kFeatSlots == turn) {
           float4& s = bins[b * kFeatSlots + (lane & (kFeatSlots - 1))];
           const float4 u = s;
           s = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
@@ -190,7 +190,8 @@ __global__ void __launch_bounds__(256) k_feat_norm(int Z, float* __restrict__ fe
     __syncthreads();
   }
   const double m = red[0] / (double)(Z * kSide);
-  for (int i = threadIdx.x; i < Z * kSide; i += blockDim.x) f[i] = m > 0 ? (float)log1p((double)f[i] / m) : 0.f;
+  const double inv = m > 0 ? 1.0 / m : 0.0;  // one division a thread: float64 bounds this pass
+  for (int i = threadIdx.x; i < Z * kSide; i += blockDim.x) f[i] = m > 0 ? (float)log1p((double)f[i] * inv) : 0.f;
 }
 
 // ---------------------------------------------------------------- phantom
