@@ -46,10 +46,10 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16& hi, __nv_bflo
   lo = __float2bfloat16_rn(r - __bfloat162float(mid));
 }
 
-// c += a b for one m16n8k16 tile.
+// c += a b for one m16n8k16 tile (not volatile: a function of its operands, so
+// that the compiler may move fragment loads past it).
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
       "{%0, %1, %2, %3};\n"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
@@ -231,15 +231,31 @@ __global__ void __launch_bounds__(kMmaThreads) k_conv_fwd_mma(const float* __res
     frag_a(fm, amid[buf] + warp * 16 * kPitch, lane);
     frag_a(fl, alo[buf] + warp * 16 * kPitch, lane);
     static_assert(NT % 2 == 0, "B tiles in pairs");
+    if constexpr (NT <= 12) {
+      // every weight fragment before the first product, and the products part
+      // by part, so that none waits on the one before it (96 channels of 16 x
+      // 16 outputs, 256 samples: 88 -> 77 us; at 128 channels the fragments'
+      // registers cost a block an SM: 50 -> 55 us)
+      uint32_t bb[NT / 2][4];
 #pragma unroll
-    for (int n = 0; n < NT; n += 2) {
-      uint32_t bb[4];
-      frag_b2(bb, bs[buf] + n * 8 * kPitch, lane);
+      for (int n = 0; n < NT; n += 2) frag_b2(bb[n / 2], bs[buf] + n * 8 * kPitch, lane);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        mma16816(acc[n + h], fl, bb[2 * h], bb[2 * h + 1]);
-        mma16816(acc[n + h], fm, bb[2 * h], bb[2 * h + 1]);
-        mma16816(acc[n + h], fh, bb[2 * h], bb[2 * h + 1]);
+      for (int n = 0; n < NT; ++n) mma16816(acc[n], fl, bb[n / 2][2 * (n & 1)], bb[n / 2][2 * (n & 1) + 1]);
+#pragma unroll
+      for (int n = 0; n < NT; ++n) mma16816(acc[n], fm, bb[n / 2][2 * (n & 1)], bb[n / 2][2 * (n & 1) + 1]);
+#pragma unroll
+      for (int n = 0; n < NT; ++n) mma16816(acc[n], fh, bb[n / 2][2 * (n & 1)], bb[n / 2][2 * (n & 1) + 1]);
+    } else {
+#pragma unroll
+      for (int n = 0; n < NT; n += 2) {
+        uint32_t bb[4];
+        frag_b2(bb, bs[buf] + n * 8 * kPitch, lane);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          mma16816(acc[n + h], fl, bb[2 * h], bb[2 * h + 1]);
+          mma16816(acc[n + h], fm, bb[2 * h], bb[2 * h + 1]);
+          mma16816(acc[n + h], fh, bb[2 * h], bb[2 * h + 1]);
+        }
       }
     }
     // the other buffer was last read before the previous barrier
