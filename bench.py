@@ -68,8 +68,8 @@ CPU_SAMPLE = (96, 256, 256)
 NCU_TRAFFIC = {
     ("field", "tf_arms"): {"bytes": 4 * (34789888 + 458295040), "digest": "a2390ea1d9919fdc"},
     ("field", "tf_psf_rows"): {"bytes": 4 * (584034048 + 423258624), "digest": "4b80f0aa1abf3e4d"},
-    ("field", "tf_yz"): {"bytes": 4 * (368307712 + 308312576), "digest": "19503de8fe03dbee"},
-    ("field", "yz_op"): {"bytes": 4 * (741899264 + 403963136), "digest": "19503de8fe03dbee"},
+    ("field", "tf_yz"): {"bytes": 4 * (368307712 + 308312576), "digest": "3e5e5d9e0b333553"},
+    ("field", "yz_op"): {"bytes": 4 * (741899264 + 403963136), "digest": "3e5e5d9e0b333553"},
 }
 
 

@@ -2,8 +2,9 @@
 // inverse z transform, in one kernel (shared by the translation units that
 // instantiate it).
 //
-// A CTA owns B adjacent x columns of one (tile, y) row of the half-spectrum
-// volumes.  The z columns of all NI input volumes are copied asynchronously
+// Up to 192 planes the stages run through registers (k_z_thru below); longer
+// columns take the shared-memory form (k_z_fused), described here.  A CTA owns
+// B adjacent x columns of one (tile, y) row of the half-spectrum volumes.  The z columns of all NI input volumes are copied asynchronously
 // into shared memory laid out [n][slot][b], so one batched transform covers
 // every volume.  The per-frequency operator then replaces, in place, the NI
 // input values at each (k, b) by the NO output values, reading the transfer
