@@ -440,7 +440,8 @@ __global__ void __launch_bounds__(ColGeom<N>::NT, (1024 / ColGeom<N>::NT) > 1 ? 
   // arms, in slot order: A, B (label-free), P (fluorescence), or
   // A, B, A' = i 2 pi eta A, B' = i 2 pi eta B (phase TF and its defocus
   // derivative), then A_tx, A_ty, A_NA (derivatives in the source parameters)
-  const bool minus = DER && a.b_even && 2 * x0 >= X;
+  // (column X/2 has no mirror: its strip is kept where the band reaches it)
+  const bool minus = DER && a.b_even && (2 * x0 > X || (2 * x0 == X && 2 * kxmax < X));
   int arm = 0;
 #pragma unroll 1
   for (int which = 0; which < (DER ? 8 : 3); ++which) {

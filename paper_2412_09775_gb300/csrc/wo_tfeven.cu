@@ -5,7 +5,8 @@
 // depend on |k_x| and |k_y| alone, phi_j = 2 pi eta z_j:
 //   - their columns k_x and -k_x are the same: only the columns 0 .. k_max of
 //     the detection band are generated, transformed along y and stored, and
-//     the row pass reads column |k_x|;
+//     the row pass reads column |k_x| (k_max reaches X/2 at critical sampling,
+//     where the rounding of k / (X p) can leave that column inside the pupil);
 //   - the source-side arm A_j = S P e^{i phi_j} needs only the columns
 //     the source reaches (the range kCntLo .. kCntHi of the pupil record), and
 //     column -k_x takes the phase factors of k_x.
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(EvenArmGeom<P>::NT, EvenArmGeom<P>::MINB) k_ar
 #if defined(WO_CHECK) && WO_CHECK
   {  // the columns +-c1 of the records and of the last arm's plane
     const long long nt = gridDim.z;
-    if (!WO_IN(c1, X / 2, 8) || !WO_IN((long long)t * N * X + (long long)(N - 1) * X + X - 1, nt * N * X, 8) ||
+    if (!WO_IN(c1, X / 2 + 1, 8) || !WO_IN((long long)t * N * X + (long long)(N - 1) * X + X - 1, nt * N * X, 8) ||
         !WO_IN((((long long)t * a.n_arms + a.n_arms - 1) * Z + j) * (long long)N * X + (long long)(N - 1) * X + X - 1,
                nt * a.n_arms * Z * (long long)N * X, 8))
       return;
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(EvenArmGeom<P>::NT, EvenArmGeom<P>::MINB) k_ar
 template <class P>
 cudaError_t launch_arms_even(const TfArgs& a, cudaStream_t s) {
   using G = EvenArmGeom<P>;
-  dim3 grid((unsigned)((a.X / 2 + G::CPC - 1) / G::CPC), (unsigned)a.Z, (unsigned)a.n_tiles);
+  dim3 grid((unsigned)((a.X / 2 + G::CPC) / G::CPC), (unsigned)a.Z, (unsigned)a.n_tiles);  // columns 0 .. X/2
   const cudaError_t attr = allow_smem(k_arms_even<P>, G::SMEM);
   if (attr != cudaSuccess) return attr;
   WO_LAUNCH("tf_arms", s, (k_arms_even<P><<<grid, G::NT, G::SMEM, s>>>(a)));
