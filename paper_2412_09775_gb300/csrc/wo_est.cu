@@ -13,6 +13,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "wo_feat.cuh"
 #include "wo_fft.cuh"
 #include "wo_internal.h"
 
@@ -73,12 +74,14 @@ __device__ __forceinline__ int freq_idx(int i, int n) { return (i < (n + 1) / 2)
 // warps an SM: 616; a slot a lane, the geometry formed by every warp: 945).
 constexpr int kFeatRows = 4, kFeatPts = 32 * kFeatRows, kFeatSlots = 8;
 
+// I: the type of an offset in a plane (feat_wide).
+template <class I>
 __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict__ spec,
                                                        const wo_optics* __restrict__ optics, int Z, int Y, int X,
                                                        float* __restrict__ feat) {
   extern __shared__ float4 sm4[];
   float4* geo = sm4;                                                      // [2][128]: ux, uy, w, bin (-1: none)
-  int2* off = reinterpret_cast<int2*>(geo + 2 * kFeatPts);                // [2][128]: the points at y and Y - y (-1: none)
+  FeatPoint<I>* off = reinterpret_cast<FeatPoint<I>*>(geo + 2 * kFeatPts);  // [2][128]: the points at y and Y - y
   const int wi = threadIdx.x / 32, lane = threadIdx.x & 31;
   float4* bins = reinterpret_cast<float4*>(off + 2 * kFeatPts) + wi * kSide * kFeatSlots;  // [64][8]
   const int r = blockIdx.x * kFeatRows + wi, t = blockIdx.y;
@@ -96,11 +99,13 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
   // float64 ones (float64 is slow on this part)
   const float inv_py = (float)(1.0 / ((double)Y * pixel)), inv_px = (float)(1.0 / ((double)X * pixel));
   const float qscale = (float)((double)kSide / cut);
-  const int points = (Y / 2 + 1) * Xh;
-  for (int p0 = 0, buf = 0; p0 < points; p0 += kFeatPts, buf ^= 1) {
+  const I points = (I)(Y / 2 + 1) * Xh;
+  int buf = 0;
+  for (I p0 = 0; p0 < points; p0 += kFeatPts, buf ^= 1) {
     {
-      const int p = p0 + threadIdx.x;
-      const int y = p / Xh, x = p - y * Xh;
+      const I p = p0 + threadIdx.x;
+      int y, x;
+      const FeatPoint<I> at = feat_point(p, Y, Xh, &y, &x);
       const float fy = (float)freq_idx(y, Y) * inv_py, fx = (float)x * inv_px;
       const float rad = sqrtf(fx * fx + fy * fy);
       const float q = rad * qscale, fl = floorf(q), fr = q - fl;
@@ -114,7 +119,7 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
       geo[buf * kFeatPts + threadIdx.x] =
           make_float4(rad > 0.f ? fx / rad : 0.f, rad > 0.f ? fy / rad : 0.f, (x == 0 || 2 * x == X) ? 1.f : 2.f,
                       __int_as_float(b));
-      off[buf * kFeatPts + threadIdx.x] = make_int2(y * Xh + x, (y > 0 && 2 * y < Y) ? (Y - y) * Xh + x : -1);
+      off[buf * kFeatPts + threadIdx.x] = at;
     }
     __syncthreads();  // (the other buffer's readers are past their loop)
     if (!row) continue;
@@ -124,12 +129,12 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
 #pragma unroll
     for (int i = 0; i < kFeatRows; ++i) {
       g[i] = geo[buf * kFeatPts + 32 * i + lane];
-      const int2 o = off[buf * kFeatPts + 32 * i + lane];
-      const bool on = __float_as_int(g[i].w) >= 0, two = on && o.y >= 0;
-      dr[i] = on ? __ldg(Dr + o.x) : zero;
-      dn[i] = on ? __ldg(Dn + o.x) : zero;
-      mr[i] = two ? __ldg(Dr + o.y) : zero;
-      mn[i] = two ? __ldg(Dn + o.y) : zero;
+      const FeatPoint<I> o = off[buf * kFeatPts + 32 * i + lane];
+      const bool on = __float_as_int(g[i].w) >= 0, two = on && o.mirror >= 0;
+      dr[i] = on ? __ldg(Dr + o.at) : zero;
+      dn[i] = on ? __ldg(Dn + o.at) : zero;
+      mr[i] = two ? __ldg(Dr + o.mirror) : zero;
+      mn[i] = two ? __ldg(Dn + o.mirror) : zero;
     }
 #pragma unroll
     for (int i = 0; i < kFeatRows; ++i) {
@@ -174,8 +179,17 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
   }
 }
 
-constexpr size_t kFeatSmem = 2 * kFeatPts * (sizeof(float4) + sizeof(int2)) +
-                             (size_t)kFeatRows * kSide * kFeatSlots * sizeof(float4);
+template <class I>
+cudaError_t launch_features(const float2* spec, const wo_optics* optics, int n, int Z, int Y, int X, float* feat,
+                            cudaStream_t s) {
+  constexpr size_t smem = 2 * kFeatPts * (sizeof(float4) + sizeof(FeatPoint<I>)) +
+                          (size_t)kFeatRows * kSide * kFeatSlots * sizeof(float4);
+  dim3 grid((unsigned)(kSide / kFeatRows), (unsigned)n);
+  const cudaError_t e = allow_smem(k_features<I>, smem);
+  if (e != cudaSuccess) return e;
+  WO_LAUNCH("est_features", s, (k_features<I><<<grid, kFeatPts, smem, s>>>(spec, optics, Z, Y, X, feat)));
+  return cudaGetLastError();
+}
 
 // One block per tile: ch0 = log(1 + P / mean P) over the Z valid rows.
 __global__ void __launch_bounds__(256) k_feat_norm(int Z, float* __restrict__ feat) {
@@ -442,11 +456,8 @@ size_t est_workspace_bytes(int B) { return est_ws(B).total; }
 
 cudaError_t est_features(const float2* spec, const wo_optics* optics, int n, int Z, int Y, int X, float* feat,
                          cudaStream_t s) {
-  dim3 grid((unsigned)(kSide / kFeatRows), (unsigned)n);
-  cudaError_t e = allow_smem(k_features, kFeatSmem);
-  if (e != cudaSuccess) return e;
-  WO_LAUNCH("est_features", s, (k_features<<<grid, kFeatPts, kFeatSmem, s>>>(spec, optics, Z, Y, X, feat)));
-  e = cudaGetLastError();
+  const cudaError_t e = feat_wide(Y, X / 2 + 1) ? launch_features<long long>(spec, optics, n, Z, Y, X, feat, s)
+                                                : launch_features<int>(spec, optics, n, Z, Y, X, feat, s);
   if (e != cudaSuccess) return e;
   WO_LAUNCH("est_feat_norm", s, (k_feat_norm<<<(unsigned)n, 256, 0, s>>>(Z, feat)));
   return cudaGetLastError();
