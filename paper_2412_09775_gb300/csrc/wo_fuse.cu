@@ -191,7 +191,13 @@ __global__ void __launch_bounds__(FuseRegGeom<P>::NT) k_z_fuse_reg(const float2*
   const long long vol = N * plane;
   const long long base = (long long)t * C * vol + col + l * plane, step = T * plane;
 #if defined(WO_CHECK) && WO_CHECK
-  if (!WO_IN((long long)t * C * vol + (C - 1) * vol + (N - 1) * plane + col, (long long)gridDim.y * C * vol, 6)) return;
+  {  // the CTA's last elements in the input and TF volumes and in the output (3D, or one plane a tile)
+    const long long end = min((long long)(blockIdx.x + 1) * G::CPC, plane) - 1, nt = gridDim.y;
+    const long long planes = op.mode == WO_MODE_3D ? N : 1;
+    if (!WO_IN((long long)t * C * vol + (C - 1) * vol + (N - 1) * plane + end, nt * C * vol, 6) ||
+        !WO_IN(((long long)t * planes + planes - 1) * plane + end, nt * planes * plane, 6))
+      return;  // uniform across the CTA
+  }
 #endif
   float2 v[E], nx[E], num[E];
   float den[E];
