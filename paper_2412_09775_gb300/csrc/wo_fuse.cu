@@ -29,45 +29,76 @@ struct FuseGeom {
 
 // Per tile: max over 3D frequencies of sum_c |H_c|^2 and max over transverse
 // frequencies of sum_k sum_c |H_c|^2 (the relative regulariser's scales in
-// 3D and 2D).  A CTA takes 32 (y, x) columns, one a lane of each of its eight
-// warps: warp g sums the planes g, g + 8, ...  (One thread a column left the chip
-// waiting on its 288 loads in turn: 4 tiles x 9 channels of 32x128x128 59.6 ->
-// 21 us, with every channel's load of a plane in flight.)
-__global__ void __launch_bounds__(256) k_fuse_stats(const float2* __restrict__ tf, int C, int Z, int Y, int Xh,
+// 3D and 2D).  Bound by the loads' latency: a lane takes one (y, x) column of
+// 32, G warps share the 32 columns (warp g the planes g, g + G, ...), and a
+// thread has 16 loads in flight: up to CM channels of 16 / CM planes.  (One thread a
+// column left the chip waiting on its 288 loads in turn: 4 tiles x 9 channels
+// of 32x128x128 66 us, now 21.)  A CTA takes column groups in turn and ends
+// in one atomic per statistic: one per warp and 32 columns, all on a few
+// words, bound banks of few channels and planes (one channel, 61 tiles of
+// 8x128x128: 93 us, now 14; 512 of 16x64x64: 212, now 32).
+constexpr int kStatsLoads = 16;
+static_assert(kStatsLoads >= kMaxFuseChannels, "a plane's channels in one batch of loads");
+
+template <int CM>
+__global__ void __launch_bounds__(256) k_fuse_stats(const float2* __restrict__ tf, int C, int Z, int Y, int Xh, int G,
                                                     float* __restrict__ stats) {
-  __shared__ float part[8][32];
-  const int t = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x / 32;
+  constexpr int U = kStatsLoads / CM;
+  __shared__ float part[8][32], red[2][8];
+  const int t = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+  const int g = warp % G;
   const long long plane = (long long)Y * Xh;
-  const long long col = (long long)blockIdx.x * 32 + lane;
-  float m3 = 0.f, s2 = 0.f;
-  if (col < plane) {
-    const float2* h = tf + (long long)t * C * Z * plane + col;
-    for (int k = g; k < Z; k += 8) {
-      float2 v[kMaxFuseChannels];  // every channel's load in flight
+  const float2* tile = tf + (long long)t * C * Z * plane;
+  float m3 = 0.f, m2 = 0.f;
+  for (long long c0 = (long long)blockIdx.x * (256 / G); c0 < plane; c0 += (long long)gridDim.x * (256 / G)) {
+    const long long col = c0 + warp / G * 32 + lane;
+    float s2 = 0.f;
+    if (col < plane) {
+      const float2* h = tile + col;
+      for (int k0 = g; k0 < Z; k0 += U * G) {
+        float2 v[U][CM];
 #pragma unroll
-      for (int c = 0; c < kMaxFuseChannels; ++c)
-        v[c] = c < C ? __ldg(h + ((long long)c * Z + k) * plane) : make_float2(0.f, 0.f);
-      float s = 0.f;
+        for (int u = 0; u < U; ++u) {
 #pragma unroll
-      for (int c = 0; c < kMaxFuseChannels; ++c) s += cabs2(v[c]);
-      m3 = fmaxf(m3, s);
-      s2 += s;
+          for (int c = 0; c < CM; ++c)
+            v[u][c] = (k0 + u * G < Z && c < C) ? __ldg(h + ((long long)c * Z + k0 + u * G) * plane)
+                                                : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          float s = 0.f;
+#pragma unroll
+          for (int c = 0; c < CM; ++c) s += cabs2(v[u][c]);
+          m3 = fmaxf(m3, s);
+          s2 += s;
+        }
+      }
     }
+    if (G > 1) {  // the column's sum over its warps
+      part[warp][lane] = s2;
+      __syncthreads();
+      s2 = 0.f;
+      if (g == 0) {
+        for (int q = 0; q < G; ++q) s2 += part[warp + q][lane];
+      }
+      __syncthreads();
+    }
+    m2 = fmaxf(m2, s2);
   }
-  part[g][lane] = s2;
-  __syncthreads();
-  s2 = 0.f;
-  if (g == 0) {
-    for (int q = 0; q < 8; ++q) s2 += part[q][lane];
-  }
+#pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    m3 = fmaxf(m3, __shfl_down_sync(0xffffffffu, m3, off));
-    s2 = fmaxf(s2, __shfl_down_sync(0xffffffffu, s2, off));
+    m3 = fmaxf(m3, __shfl_xor_sync(0xffffffffu, m3, off));
+    m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, off));
   }
-  // values are >= 0: integer order equals float order
   if (lane == 0) {
-    if (m3 > 0.f) atomicMax(reinterpret_cast<int*>(stats) + 2 * t, __float_as_int(m3));
-    if (s2 > 0.f) atomicMax(reinterpret_cast<int*>(stats) + 2 * t + 1, __float_as_int(s2));
+    red[0][warp] = m3;
+    red[1][warp] = m2;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {  // values are >= 0: integer order equals float order
+    float m = 0.f;
+    for (int q = 0; q < 8; ++q) m = fmaxf(m, red[threadIdx.x][q]);
+    if (m > 0.f) atomicMax(reinterpret_cast<int*>(stats) + 2 * t + threadIdx.x, __float_as_int(m));
   }
 }
 
@@ -285,8 +316,19 @@ cudaError_t fuse_stats(const float2* tf, int n_tiles, int C, int Z, int Y, int X
   cudaError_t e = cudaMemsetAsync(stats, 0, (size_t)n_tiles * 2 * sizeof(float), s);
   if (e != cudaSuccess) return e;
   const long long plane = (long long)Y * Xh;
-  dim3 grid((unsigned)((plane + 31) / 32), (unsigned)n_tiles);
-  WO_LAUNCH("fuse_stats", s, (k_fuse_stats<<<grid, 256, 0, s>>>(tf, C, Z, Y, Xh, stats)));
+  // warps a column: enough planes each to fill a thread's loads; CTAs: about
+  // two waves of eight an SM over the batch (more only add atomics)
+  const int cm = C == 1 ? 1 : C <= 4 ? 4 : kStatsLoads;
+  int G = 8;
+  while (G > 1 && G * (kStatsLoads / cm) > Z) G /= 2;
+  const long long groups = (plane + 256 / G - 1) / (256 / G), want = (2 * 8 * 152 + n_tiles - 1) / n_tiles;
+  dim3 grid((unsigned)(groups < want ? groups : want), (unsigned)n_tiles);
+  auto run = [&](auto kernel) {
+    WO_LAUNCH("fuse_stats", s, (kernel<<<grid, 256, 0, s>>>(tf, C, Z, Y, Xh, G, stats)));
+  };
+  if (cm == 1) run(k_fuse_stats<1>);
+  else if (cm == 4) run(k_fuse_stats<4>);
+  else run(k_fuse_stats<kStatsLoads>);
   return cudaGetLastError();
 }
 
