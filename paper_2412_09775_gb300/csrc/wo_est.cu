@@ -74,8 +74,13 @@ __device__ __forceinline__ int freq_idx(int i, int n) { return (i < (n + 1) / 2)
 // warps an SM: 616; a slot a lane, the geometry formed by every warp: 945).
 constexpr int kFeatRows = 4, kFeatPts = 32 * kFeatRows, kFeatSlots = 8;
 
-// I: the type of an offset in a plane (feat_wide).
-template <class I>
+// I: the type of an offset in a plane (feat_wide).  RPC: rows a CTA, four, or
+// one while those CTAs all fit the chip at once: its four warps then take 32
+// points each of every 128, so that a row's walk is a quarter as long (one
+// tile of 48x128x128 70 -> 38 us, 16 78 -> 76; 64 182, with one row a CTA 245).
+// CTAs whose rows are all past the stack only write zeros (1024 tiles of
+// 4x32x32, 60 of 64 rows past it: 263 -> 43 us).
+template <class I, int RPC>
 __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict__ spec,
                                                        const wo_optics* __restrict__ optics, int Z, int Y, int X,
                                                        float* __restrict__ feat) {
@@ -84,8 +89,16 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
   FeatPoint<I>* off = reinterpret_cast<FeatPoint<I>*>(geo + 2 * kFeatPts);  // [2][128]: the points at y and Y - y
   const int wi = threadIdx.x / 32, lane = threadIdx.x & 31;
   float4* bins = reinterpret_cast<float4*>(off + 2 * kFeatPts) + wi * kSide * kFeatSlots;  // [64][8]
-  const int r = blockIdx.x * kFeatRows + wi, t = blockIdx.y;
+  static_assert(RPC == kFeatRows || RPC == 1, "a warp a row, or every warp on one");
+  constexpr int PL = RPC;  // points a lane takes of every 128
+  const int r = blockIdx.x * RPC + (RPC > 1 ? wi : 0), t = blockIdx.y;
   const int Xh = X / 2 + 1;
+  if ((int)blockIdx.x * RPC >= Z) {
+    float* out = feat + (long long)t * 3 * kSide * kSide + blockIdx.x * RPC * kSide;
+    for (int e = threadIdx.x; e < 3 * RPC * kSide; e += kFeatPts)
+      out[e / (RPC * kSide) * kSide * kSide + e % (RPC * kSide)] = 0.f;
+    return;  // uniform across the CTA
+  }
   const double pixel = optics[t].pixel_um, cut = 2.0 * optics[t].na_det / optics[t].lambda_um;
   for (int b = lane; b < kSide * kFeatSlots; b += 32) bins[b] = make_float4(0.f, 0.f, 0.f, 0.f);
   const long long plane = (long long)Y * Xh;
@@ -123,13 +136,14 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
     }
     __syncthreads();  // (the other buffer's readers are past their loop)
     if (!row) continue;
-    float2 dr[kFeatRows], dn[kFeatRows], mr[kFeatRows], mn[kFeatRows];
-    float4 g[kFeatRows];
+    float2 dr[PL], dn[PL], mr[PL], mn[PL];
+    float4 g[PL];
     const float2 zero = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < kFeatRows; ++i) {
-      g[i] = geo[buf * kFeatPts + 32 * i + lane];
-      const FeatPoint<I> o = off[buf * kFeatPts + 32 * i + lane];
+    for (int i = 0; i < PL; ++i) {
+      const int e = buf * kFeatPts + 32 * (RPC > 1 ? i : wi) + lane;
+      g[i] = geo[e];
+      const FeatPoint<I> o = off[e];
       const bool on = __float_as_int(g[i].w) >= 0, two = on && o.mirror >= 0;
       dr[i] = on ? __ldg(Dr + o.at) : zero;
       dn[i] = on ? __ldg(Dn + o.at) : zero;
@@ -137,7 +151,7 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
       mn[i] = two ? __ldg(Dn + o.mirror) : zero;
     }
 #pragma unroll
-    for (int i = 0; i < kFeatRows; ++i) {
+    for (int i = 0; i < PL; ++i) {
       const int b = __float_as_int(g[i].w);
       const float pr = cabs2(dr[i]), pm = cabs2(mr[i]);
       // Im of D_next conj(D_r), at y and Y - y
@@ -162,16 +176,20 @@ __global__ void __launch_bounds__(kFeatPts) k_features(const float2* __restrict_
   }
   if (r >= kSide) return;
   float* out = feat + (long long)t * 3 * kSide * kSide + (long long)r * kSide;
-  __syncwarp();
-  for (int b = lane; b < kSide; b += 32) {
+  if (RPC > 1) __syncwarp();
+  else __syncthreads();
+  bins -= RPC > 1 ? 0 : wi * kSide * kFeatSlots;
+  for (int b = RPC > 1 ? lane : threadIdx.x; b < kSide; b += RPC > 1 ? 32 : kFeatPts) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int w = 0; w < kFeatRows / RPC; ++w) {
 #pragma unroll 8
-    for (int l = 0; l < kFeatSlots; ++l) {  // each lane starts at another slot: distinct banks
-      const float4 u = bins[b * kFeatSlots + ((l + lane) & (kFeatSlots - 1))];
-      v.x += u.x;
-      v.y += u.y;
-      v.z += u.z;
-      v.w += u.w;
+      for (int l = 0; l < kFeatSlots; ++l) {  // each lane starts at another slot: distinct banks
+        const float4 u = bins[(w * kSide + b) * kFeatSlots + ((l + lane) & (kFeatSlots - 1))];
+        v.x += u.x;
+        v.y += u.y;
+        v.z += u.z;
+        v.w += u.w;
+      }
     }
     out[b] = v.x;
     out[kSide * kSide + b] = v.y > 0.f ? v.z / v.y : 0.f;
@@ -184,11 +202,16 @@ cudaError_t launch_features(const float2* spec, const wo_optics* optics, int n, 
                             cudaStream_t s) {
   constexpr size_t smem = 2 * kFeatPts * (sizeof(float4) + sizeof(FeatPoint<I>)) +
                           (size_t)kFeatRows * kSide * kFeatSlots * sizeof(float4);
-  dim3 grid((unsigned)(kSide / kFeatRows), (unsigned)n);
-  const cudaError_t e = allow_smem(k_features<I>, smem);
-  if (e != cudaSuccess) return e;
-  WO_LAUNCH("est_features", s, (k_features<I><<<grid, kFeatPts, smem, s>>>(spec, optics, Z, Y, X, feat)));
-  return cudaGetLastError();
+  auto run = [&](auto kernel, int rows) {
+    const cudaError_t e = allow_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((unsigned)(kSide / rows), (unsigned)n);
+    WO_LAUNCH("est_features", s, (kernel<<<grid, kFeatPts, smem, s>>>(spec, optics, Z, Y, X, feat)));
+    return cudaGetLastError();
+  };
+  // (five CTAs an SM by shared memory)
+  if ((long long)n * Z <= 5 * 152) return run(k_features<I, 1>, 1);
+  return run(k_features<I, kFeatRows>, kFeatRows);
 }
 
 // One block per tile: ch0 = log(1 + P / mean P) over the Z valid rows.
