@@ -381,6 +381,11 @@ __global__ void __launch_bounds__(ZThruGeom<N, NI, NO>::NT, ZThruGeom<N, NI, NO>
 }
 
 // 2D: out[t][p][y][x] = (sum_k H_k^H H_k + lam I)^-1 sum_k H_k^H D_k per mode.
+// Bound by the latency of the transfer functions' loads after the transform:
+// two planes' loads go out together.  Left to itself the compiler unrolled the
+// loop or not, by length and kinds, from one version of the code around it to
+// the next (two kinds, 45 x 32x128x128: 58 or 74 us; with pairs 56; three
+// kinds, 91 x 16x128x128: 110 or 127; with pairs 97).
 template <int N, int NI>
 __global__ void __launch_bounds__(ZGeom<N, NI>::NT, ZGeom<N, NI>::MINB)
     k_z_solve2d(const float2* __restrict__ in, float2* __restrict__ out, const float2* __restrict__ tf, ZOp op,
@@ -428,31 +433,43 @@ __global__ void __launch_bounds__(ZGeom<N, NI>::NT, ZGeom<N, NI>::MINB)
   for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
   // columns outside the support disk hold only the TFs' rounding noise: zero out
   if (b < w && !outside_support(op.stats + (long long)tt * 8, y, Y, x0 + b, 2 * (Xh - 1))) {
-    for (int k = kk; k < N; k += KK) {
-      const float2* cell = buf + k * NI * B + b;
-      const bool dc = op.zero_dc && k == 0 && y == 0 && (x0 + b) == 0;
-      const float2* h = tf + ((long long)tt * op.n_tf * N + k) * zs + col + b;
-      if (L > 0) {
-        const float2 d = dc ? make_float2(0.f, 0.f) : cell[op.lf_chan * B];
-        const float2 h0 = __ldg(h);
-        acc[0] += cabs2(h0);
-        const float2 r0 = cmulc(h0, d);
-        acc[4] += r0.x; acc[5] += r0.y;
-        if (L > 1) {
-          const float2 h1 = __ldg(h + vol);
-          acc[1] += cabs2(h1);
-          const float2 m01 = cmulc(h0, h1);
-          acc[2] += m01.x; acc[3] += m01.y;
-          const float2 r1 = cmulc(h1, d);
-          acc[6] += r1.x; acc[7] += r1.y;
-        }
+    constexpr int U = 2;  // planes whose transfer functions are on their way together
+    for (int k0 = kk; k0 < N; k0 += U * KK) {
+      float2 h0[U], h1[U], hf[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * KK;
+        const bool ok = N % (U * KK) == 0 || k < N;
+        const float2* h = tf + ((long long)tt * op.n_tf * N + k) * zs + col + b;
+        h0[u] = ok && L > 0 ? __ldg(h) : make_float2(0.f, 0.f);
+        h1[u] = ok && L > 1 ? __ldg(h + vol) : make_float2(0.f, 0.f);
+        hf[u] = ok && op.has_fl ? __ldg(h + L * vol) : make_float2(0.f, 0.f);
       }
-      if (op.has_fl) {
-        const float2 d = dc ? make_float2(0.f, 0.f) : cell[op.fl_chan * B];
-        const float2 hf = __ldg(h + L * vol);
-        acc[8] += cabs2(hf);
-        const float2 rf = cmulc(hf, d);
-        acc[9] += rf.x; acc[10] += rf.y;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * KK;
+        if (N % (U * KK) != 0 && k >= N) break;
+        const float2* cell = buf + k * NI * B + b;
+        const bool dc = op.zero_dc && k == 0 && y == 0 && (x0 + b) == 0;
+        if (L > 0) {
+          const float2 d = dc ? make_float2(0.f, 0.f) : cell[op.lf_chan * B];
+          acc[0] += cabs2(h0[u]);
+          const float2 r0 = cmulc(h0[u], d);
+          acc[4] += r0.x; acc[5] += r0.y;
+          if (L > 1) {
+            acc[1] += cabs2(h1[u]);
+            const float2 m01 = cmulc(h0[u], h1[u]);
+            acc[2] += m01.x; acc[3] += m01.y;
+            const float2 r1 = cmulc(h1[u], d);
+            acc[6] += r1.x; acc[7] += r1.y;
+          }
+        }
+        if (op.has_fl) {
+          const float2 d = dc ? make_float2(0.f, 0.f) : cell[op.fl_chan * B];
+          acc[8] += cabs2(hf[u]);
+          const float2 rf = cmulc(hf[u], d);
+          acc[9] += rf.x; acc[10] += rf.y;
+        }
       }
     }
   }
