@@ -2,11 +2,12 @@
 // inverse z transform, in one kernel (shared by the translation units that
 // instantiate it).
 //
-// Up to 192 planes the stages run through registers (k_z_thru below); longer
-// columns take the shared-memory form (k_z_fused), described here.  A CTA owns
-// B adjacent x columns of one (tile, y) row of the half-spectrum volumes.  The z columns of all NI input volumes are copied asynchronously
-// into shared memory laid out [n][slot][b], so one batched transform covers
-// every volume.  The per-frequency operator then replaces, in place, the NI
+// Up to 192 planes the stages run through registers (k_z_thru below; z_thru()
+// says where); the other lengths take the shared-memory form (k_z_fused),
+// described here.  A CTA owns B adjacent x columns of one (tile, y) row of the
+// half-spectrum volumes.  The z columns of all NI input volumes are copied
+// asynchronously into shared memory laid out [n][slot][b], so one batched
+// transform covers every volume.  The per-frequency operator then replaces, in place, the NI
 // input values at each (k, b) by the NO output values, reading the transfer
 // functions once (coalesced along x); the NO outputs are transformed back in
 // one batch and stored.  The operators are
@@ -23,9 +24,8 @@
 
 namespace wo {
 
-// Columns per CTA of the z kernels: 16 while the tile stays within 32 KB,
-// else the widest that fits 64 KB.  At 96 planes and three volumes 8 columns
-// (more CTAs resident per SM) measured faster than 16 and 4.
+// Columns per CTA of the shared-memory z kernels: 16 while the tile stays
+// within 32 KB, else the widest that fits 64 KB.
 __host__ __device__ constexpr int z_cols(int N, int NV) {
   return (NV * N * 16 * 8 <= 32 * 1024) ? 16
          : (NV * N * 8 * 8 <= 64 * 1024) ? 8
@@ -510,25 +510,34 @@ __global__ void __launch_bounds__(ZGeom<N, NI>::NT, ZGeom<N, NI>::MINB)
   }
 }
 
+// Where the columns go through registers: up to 192 planes (longer ones have
+// only been measured in shared memory).  One volume of 12 or 24 planes stays in
+// shared memory: the first stage, three butterflies a column, then leaves up to
+// five threads in eight of a CTA without a load (24 planes, 61 x 128x128: 65 us,
+// through registers 88; 15 x 256x256: 59, 82; 12 planes of 256x256: 56, 62).
+// With two or three volumes every thread loads.
+template <int N, int NI, int NO>
+constexpr bool z_thru() {
+  return N > 1 && N <= 192 && !(NI == 1 && NO == 1 && (N == 12 || N == 24));
+}
+
 template <int N, int NI, int NO>
 cudaError_t launch_z_fused(const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles, int Y, int Xh,
                            cudaStream_t s) {
-  constexpr int NV = NI > NO ? NI : NO;
-  // one plane has no transform; past 192 the last stage's butterflies outnumber a CTA's threads
-  if constexpr (N > 1 && N <= 192) {
+  if constexpr (z_thru<N, NI, NO>()) {
     using G = ZThruGeom<N, NI, NO>;
     const cudaError_t attr = allow_smem(k_z_thru<N, NI, NO>, G::SMEM);
     if (attr != cudaSuccess) return attr;
     dim3 grid((unsigned)((Y * Xh + G::B - 1) / G::B), (unsigned)n_tiles);
     WO_LAUNCH("z_fused", s, (k_z_thru<N, NI, NO><<<grid, G::NT, G::SMEM, s>>>(in, out, tf, op, Y, Xh)));
-    return cudaGetLastError();
+  } else {
+    using G = ZGeom<N, (NI > NO ? NI : NO)>;
+    const cudaError_t attr = allow_smem(k_z_fused<N, NI, NO>, G::SMEM_TF);
+    if (attr != cudaSuccess) return attr;
+    dim3 grid((unsigned)((Xh + G::B - 1) / G::B), (unsigned)Y, (unsigned)n_tiles);
+    const size_t smem = G::smem_tf(op.n_tf < 3 ? op.n_tf : 3);
+    WO_LAUNCH("z_fused", s, (k_z_fused<N, NI, NO><<<grid, G::NT, smem, s>>>(in, out, tf, op, Y, Xh)));
   }
-  using G = ZGeom<N, NV>;
-  const cudaError_t attr = allow_smem(k_z_fused<N, NI, NO>, G::SMEM_TF);
-  if (attr != cudaSuccess) return attr;
-  dim3 grid((unsigned)((Xh + G::B - 1) / G::B), (unsigned)Y, (unsigned)n_tiles);
-  const size_t smem = G::smem_tf(op.n_tf < 3 ? op.n_tf : 3);
-  WO_LAUNCH("z_fused", s, (k_z_fused<N, NI, NO><<<grid, G::NT, smem, s>>>(in, out, tf, op, Y, Xh)));
   return cudaGetLastError();
 }
 
