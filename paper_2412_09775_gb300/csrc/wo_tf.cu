@@ -689,11 +689,13 @@ __global__ void __launch_bounds__(ZGeom<N, NK>::NT, ZGeom<N, NK>::MINB) k_tf_zpa
 
 // The z pass by the scheme of k_z_thru (wo_zops.cuh): the first stage loads
 // from global memory, the last one keeps every kind's values of its
-// frequencies in registers, forms the maxima and stores.  The columns of a
-// tile in the order of memory; those with k_x >= x_cols are left as they are.
+// frequencies in registers, forms the maxima and stores.  The columns with
+// k_x >= x_cols are left as they are.  A CTA takes B columns of a row-major walk
+// over the first `cols` of every row: x_cols, or the whole row, whose lines
+// are whole (zpass_cols below); CTAs without a column to transform leave.
 // Three kinds, 96x512x257: 149 -> 131 us.
 template <int N, int NK>
-__global__ void __launch_bounds__(ZThruGeom<N, NK, NK>::NT, ZThruGeom<N, NK, NK>::MINB) k_tf_zthru(TfArgs a) {
+__global__ void __launch_bounds__(ZThruGeom<N, NK, NK>::NT, ZThruGeom<N, NK, NK>::MINB) k_tf_zthru(TfArgs a, int cols) {
   using G = ZThruGeom<N, NK, NK>;
   constexpr int B = G::B, NT = G::NT, RL = G::RL, ML = G::ML, S = G::S;
   extern __shared__ float2 sm[];
@@ -701,13 +703,21 @@ __global__ void __launch_bounds__(ZThruGeom<N, NK, NK>::NT, ZThruGeom<N, NK, NK>
   float2* buf = sm + N;
   float* red = reinterpret_cast<float*>(sm + G::SMEM / sizeof(float2));  // [2][NT]
   const int Xh = a.X / 2 + 1, zs = a.Y * Xh;
-  const int t = blockIdx.y, b = threadIdx.x % B, k0 = threadIdx.x / B, c = blockIdx.x * B + b;
-  const bool live = c < zs && c % Xh < a.x_cols;
+  const int t = blockIdx.y, b = threadIdx.x % B, k0 = threadIdx.x / B, e = blockIdx.x * B + b;
+  const int y = e / cols, x = e - y * cols, c = y * Xh + x;
+  const bool live = y < a.Y && x < a.x_cols;
+  {  // every column past x_cols, in one row (uniform across the CTA)
+    const int x0 = (int)(blockIdx.x * B) % cols;
+    if (x0 >= a.x_cols && x0 + B <= cols) return;
+  }
   const long long vol = (long long)N * zs;
 #if defined(WO_CHECK) && WO_CHECK
-  if (!WO_IN(((long long)t * NK + NK - 1) * vol + (long long)(N - 1) * zs + min((int)(blockIdx.x + 1) * B, zs) - 1,
-             (long long)gridDim.y * NK * vol, 6))
-    return;  // uniform across the CTA
+  {  // the CTA's last column
+    const int last = min((int)(blockIdx.x + 1) * B, a.Y * cols) - 1;
+    if (!WO_IN(((long long)t * NK + NK - 1) * vol + (long long)(N - 1) * zs + last / cols * Xh + last % cols,
+               (long long)gridDim.y * NK * vol, 6))
+      return;  // uniform across the CTA
+  }
 #endif
   float2* base = a.tf + (long long)t * NK * vol + c;
   const float2 zero = make_float2(0.f, 0.f);
@@ -863,24 +873,45 @@ cudaError_t tf_psf_rows(const TfArgs& a, cudaStream_t s) {
   }
 }
 
+// Where the columns go through registers: up to 192 planes, but not 128, whose
+// last stage is of radix 2 (two kinds, 9 x 128x128: 82 us in shared memory, 108
+// through registers; three, 1 x 512x512: 199, 210), nor two kinds of 192 (89 and 91).
+template <int N, int NK>
+constexpr bool zpass_thru() {
+  return N > 1 && N <= 192 && N != 128 && !(N == 192 && NK < 3);
+}
+
+// Columns of a row that the CTAs walk.  Leaving out those past x_cols pays
+// where they are many (a quarter; three kinds, 3 x 96x256x256 at an eighth of
+// the pixel: 80 -> 21 us), and always where 16 or 32 columns a CTA meet a last
+// stage of radix 2 or 3 (12, 16, 24, 48 planes: two kinds, 19 x 16x256x256, an
+// eighth of the row: 69 -> 63 us).  Otherwise the broken lines cost more (three
+// kinds, 19 x 64x128x128: 77 -> 84).
+template <class G>
+int zpass_cols(const TfArgs& a) {
+  const int Xh = a.X / 2 + 1;
+  return 4 * a.x_cols <= 3 * Xh || ((G::B == 16 || G::B == 32) && G::RL <= 3) ? a.x_cols : Xh;
+}
+
 template <int N, int NK>
 static cudaError_t launch_zpass(const TfArgs& a, cudaStream_t s) {
-  if constexpr (N > 1 && N <= 192) {  // (the lengths of k_z_thru)
+  if (a.x_cols <= 0) return cudaSuccess;
+  if constexpr (zpass_thru<N, NK>()) {
     using G = ZThruGeom<N, NK, NK>;
     constexpr size_t smem = G::SMEM + (size_t)2 * G::NT * sizeof(float);
     const cudaError_t attr = allow_smem(k_tf_zthru<N, NK>, smem);
     if (attr != cudaSuccess) return attr;
-    if (a.x_cols <= 0) return cudaSuccess;
-    dim3 grid((unsigned)((a.Y * (a.X / 2 + 1) + G::B - 1) / G::B), (unsigned)a.n_tiles);
-    WO_LAUNCH("tf_zpass", s, (k_tf_zthru<N, NK><<<grid, G::NT, smem, s>>>(a)));
-    return cudaGetLastError();
+    const int cols = zpass_cols<G>(a);
+    dim3 grid((unsigned)((a.Y * cols + G::B - 1) / G::B), (unsigned)a.n_tiles);
+    WO_LAUNCH("tf_zpass", s, (k_tf_zthru<N, NK><<<grid, G::NT, smem, s>>>(a, cols)));
+  } else {
+    using G = ZGeom<N, NK>;
+    const size_t smem = G::SMEM + (size_t)G::NT * 2 * sizeof(float);
+    const cudaError_t attr = allow_smem(k_tf_zpass<N, NK>, smem);
+    if (attr != cudaSuccess) return attr;
+    dim3 grid((unsigned)((a.x_cols + G::B - 1) / G::B), (unsigned)a.Y, (unsigned)a.n_tiles);
+    WO_LAUNCH("tf_zpass", s, (k_tf_zpass<N, NK><<<grid, G::NT, smem, s>>>(a)));
   }
-  using G = ZGeom<N, NK>;
-  const size_t smem = G::SMEM + (size_t)G::NT * 2 * sizeof(float);
-  const cudaError_t attr = allow_smem(k_tf_zpass<N, NK>, smem);
-  if (attr != cudaSuccess) return attr;
-  dim3 grid((unsigned)((a.x_cols + G::B - 1) / G::B), (unsigned)a.Y, (unsigned)a.n_tiles);
-  WO_LAUNCH("tf_zpass", s, (k_tf_zpass<N, NK><<<grid, G::NT, smem, s>>>(a)));
   return cudaGetLastError();
 }
 
