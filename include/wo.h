@@ -574,8 +574,9 @@ enum { WO_PASS_COLS = 0 };
  * points: WO_ENGINE_SMEM (rows staged in shared memory, Stockham stages) or
  * WO_ENGINE_HYBRID (each row held by T lanes of one warp straight from global
  * memory, register-resident four-step transform, the Hermitian split by warp
- * shuffles; n = 32, 48, 64, 96, 128, 192, 256, 512; the default where it
- * exists). */
+ * shuffles; n = 32, 48, 64, 96, 128, 192, 256, 384, 512; the default where it
+ * exists).  The passes that read tiles from a field or blend into one have
+ * the register form alone, without n = 384. */
 enum { WO_PASS_ROWS = 1 };
 /* WO_PASS_RECON: the phase-only 3D reconstruction (wo_reconstruct,
  * wo_reconstruct_shared_tf with kinds WO_TF_PHASE, optionally with

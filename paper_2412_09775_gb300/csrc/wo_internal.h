@@ -244,7 +244,8 @@ inline cudaError_t plane_xy_inv(int X, int Y, float2* in, float* out, long long 
   return plane_xy_inv(X, Y, in, out, nplanes, scale, bg, s, xy_engine(X, Y));
 }
 int rows_engine(int n);  // engine of the x passes for n complex points (wo_rowsreg.cu: HYBRID)
-bool rows_reg_supported(int N);
+bool rows_reg_supported(int N);     // the x passes of tiles and fields too
+bool rows_engine_supported(int N);  // the plain x passes
 cudaError_t rows_r2c_reg(int N, const float* in, float2* out, long long nrows, RowBg bg, cudaStream_t s);
 // The tiles of a field as the rows' source (wo_rowsreg.cu): tile t = (ty, tx)
 // of a tiles_y x tiles_x grid covers field rows ty*core - halo .. and

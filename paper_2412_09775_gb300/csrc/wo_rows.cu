@@ -156,16 +156,14 @@ static cudaError_t launch_c2r(const float2* in, float* out, long long nrows, flo
 
 cudaError_t rows_r2c(int N, const float* in, float2* out, long long nrows, RowBg bg, cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  // rows of 768 samples: in registers only (the shared-memory rows took
-  // longer both ways: 18432 rows, R2C 82 -> 48 us, C2R 77 -> 51 us)
-  if (N == 384 || rows_engine(N) == WO_ENGINE_HYBRID) return rows_r2c_reg(N, in, out, nrows, bg, s);
+  if (rows_engine(N) == WO_ENGINE_HYBRID) return rows_r2c_reg(N, in, out, nrows, bg, s);
   switch (N) {
 #define WO_CASE(n) \
   case n:          \
     return launch_r2c<n>(in, out, nrows, bg, s);
     WO_CASE(1) WO_CASE(2) WO_CASE(3) WO_CASE(4) WO_CASE(6) WO_CASE(8) WO_CASE(12) WO_CASE(16)
     WO_CASE(24) WO_CASE(32) WO_CASE(48) WO_CASE(64) WO_CASE(96) WO_CASE(128) WO_CASE(192)
-    WO_CASE(256) WO_CASE(512) WO_CASE(768) WO_CASE(1024)
+    WO_CASE(256) WO_CASE(384) WO_CASE(512) WO_CASE(768) WO_CASE(1024)
 #undef WO_CASE
     default:
       return cudaErrorInvalidValue;
@@ -175,14 +173,14 @@ cudaError_t rows_r2c(int N, const float* in, float2* out, long long nrows, RowBg
 cudaError_t rows_c2r(int N, const float2* in, float* out, long long nrows, float scale, RowBg bg,
                      cudaStream_t s) {
   if (nrows <= 0) return cudaSuccess;
-  if (N == 384 || rows_engine(N) == WO_ENGINE_HYBRID) return rows_c2r_reg(N, in, out, nrows, scale, bg, s);
+  if (rows_engine(N) == WO_ENGINE_HYBRID) return rows_c2r_reg(N, in, out, nrows, scale, bg, s);
   switch (N) {
 #define WO_CASE(n) \
   case n:          \
     return launch_c2r<n>(in, out, nrows, scale, bg, s);
     WO_CASE(1) WO_CASE(2) WO_CASE(3) WO_CASE(4) WO_CASE(6) WO_CASE(8) WO_CASE(12) WO_CASE(16)
     WO_CASE(24) WO_CASE(32) WO_CASE(48) WO_CASE(64) WO_CASE(96) WO_CASE(128) WO_CASE(192)
-    WO_CASE(256) WO_CASE(512) WO_CASE(768) WO_CASE(1024)
+    WO_CASE(256) WO_CASE(384) WO_CASE(512) WO_CASE(768) WO_CASE(1024)
 #undef WO_CASE
     default:
       return cudaErrorInvalidValue;

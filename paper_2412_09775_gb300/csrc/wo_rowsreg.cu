@@ -398,7 +398,10 @@ cudaError_t launch_c2r_reg(const float2* in, float* out, long long nrows, float 
 
 }  // namespace
 
-// The lengths whose engine the schedule may choose (and the tile passes take).
+// The lengths of the passes that read and write tiles, fields and kx-major
+// spectra; the plain x passes also have 384 points (Row384).
+bool rows_engine_supported(int N) { return N == 384 || rows_reg_supported(N); }
+
 bool rows_reg_supported(int N) {
   return N == 32 || N == 48 || N == 64 || N == 96 || N == 128 || N == 192 || N == 256 || N == 512;
 }

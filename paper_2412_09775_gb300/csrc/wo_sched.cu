@@ -81,11 +81,12 @@ int cols_engine(int n) {
 }
 
 int rows_engine(int n) {
-  if (n < 1 || n > kMaxLen || !rows_reg_supported(n)) return WO_ENGINE_SMEM;
+  if (n < 1 || n > kMaxLen || !rows_engine_supported(n)) return WO_ENGINE_SMEM;
   const int e = g_rows_engine[n].load(std::memory_order_relaxed);
   if (e == WO_ENGINE_SMEM || e == WO_ENGINE_HYBRID) return e;
   // default: the register rows, faster on the workloads' x passes (256 and 96
-  // points: 0.127 -> 0.087 ms and 0.152 -> 0.112 ms on the widefield step)
+  // points: 0.127 -> 0.087 ms and 0.152 -> 0.112 ms on the widefield step; 384
+  // points, 18432 rows: 0.082 -> 0.048 ms forward, 0.077 -> 0.051 ms back)
   return WO_ENGINE_HYBRID;
 }
 
@@ -169,7 +170,7 @@ static int tune_rows(int n, long long rows, float2* scratch, cudaStream_t s) {
   float* real = reinterpret_cast<float*>(scratch);
   float2* half = scratch + (size_t)rows * n;  // after the 2n real samples of every row
   const RowBg none{};
-  return tune_entry(g_rows_engine[n], WO_ENGINE_HYBRID, rows_reg_supported(n), s, [&](int) {
+  return tune_entry(g_rows_engine[n], WO_ENGINE_HYBRID, rows_engine_supported(n), s, [&](int) {
     cudaError_t e = rows_r2c(n, real, half, rows, none, s);
     if (e != cudaSuccess) return e;
     return rows_c2r(n, half, real, rows, 1.0f, none, s);
@@ -196,7 +197,7 @@ wo_status wo_schedule_set(int pass, int n, int engine) {
     g_xy_engine[n].store(engine, std::memory_order_relaxed);
     return WO_OK;
   }
-  const bool hyb_ok = pass == WO_PASS_COLS ? cols_hyb_supported(n) : rows_reg_supported(n);
+  const bool hyb_ok = pass == WO_PASS_COLS ? cols_hyb_supported(n) : rows_engine_supported(n);
   if (engine == WO_ENGINE_HYBRID && !hyb_ok) return WO_ERR_UNSUPPORTED_SIZE;
   (pass == WO_PASS_COLS ? g_cols_engine : g_rows_engine)[n].store(engine, std::memory_order_relaxed);
   return WO_OK;
@@ -238,7 +239,7 @@ wo_status wo_autotune(int n_tiles, int Z, int Y, int X, unsigned kinds, void* d_
   if (Z > 1 && Z != Y && tune_cols(Z, Y * Xh, vols, scratch, s) < 0) return WO_ERR_CUDA;
   // x passes: the rows of the same volumes (2n real samples in, n+1 bins out
   // per row fit the volumes' half spectra twice over)
-  if (rows_reg_supported(X / 2) && tune_rows(X / 2, vols * Z * Y, scratch, s) < 0) return WO_ERR_CUDA;
+  if (rows_engine_supported(X / 2) && tune_rows(X / 2, vols * Z * Y, scratch, s) < 0) return WO_ERR_CUDA;
   // fused x-y planes (the same volumes' planes, real and half spectrum side by side)
   if (xy_supported(X, Y) && tune_xy(X, vols * Z, scratch, s) < 0) return WO_ERR_CUDA;
   return cudaStreamSynchronize(s) == cudaSuccess ? WO_OK : WO_ERR_CUDA;
