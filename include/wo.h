@@ -559,13 +559,17 @@ wo_status wo_thin_phantom(const float *d_params, int n_tiles, int n_spheres, int
  * depend on the engine beyond float32 rounding.
  * wo_schedule_set: WO_ERR_ARG on a bad pass, length or engine,
  * WO_ERR_UNSUPPORTED_SIZE for an engine that lacks the length.
- * wo_schedule_get: the engine in use for (pass, n), -1 on bad arguments.
+ * wo_schedule_get: the engine in use for (pass, n), -1 on bad arguments;
+ * where the built-in choice depends on the batch (WO_PASS_XY, n = 64), that of
+ * large batches.  wo_schedule_set with that answer pins it for every batch;
+ * WO_ENGINE_DEFAULT restores the built-in rule.
  * wo_autotune: times every engine of the column transforms that an entry
  * point on these shapes launches (lengths Y and Z, batches as large as the
  * workspace allows up to three volumes per tile) and of the x passes (X/2
  * points, the rows of the same volumes), on the workspace (its
- * contents are destroyed), and keeps the fastest in the table (the non-default
- * engine only when at least 2 % faster).  It waits for
+ * contents are destroyed), and keeps the fastest in the table (another than
+ * the built-in engine of these shapes only when at least 2 % faster; where the
+ * built-in one stays, the entry returns to the built-in rule).  It waits for
  * the stream (it measures with events), so it is not for graph capture; run
  * it once before capturing.  The table is process-wide. */
 enum { WO_PASS_COLS = 0 };
@@ -602,8 +606,11 @@ enum { WO_PASS_RECON = 2 };
  * columns along y, so the intermediate spectrum never goes to memory;
  * n = 64, 128, 192).  The default is WO_ENGINE_SMEM: the fused kernels hold
  * a plane tile of about 109 KB per CTA (192 x 192), two CTAs per SM, and
- * measured slower on the 256-tile field; wo_autotune picks them where they
- * are faster.  Results agree to float32 rounding. */
+ * measured slower on the 256-tile field; but the operators (wo_forward,
+ * wo_forward_adjoint, wo_reconstruct and its shared-TF and static forms) run
+ * a direction's pass over up to 768 planes of 64 x 64 on the fused kernels,
+ * which save such a call two launches of five.  wo_autotune picks either
+ * where it is faster.  Results agree to float32 rounding. */
 enum { WO_PASS_XY = 3 };
 enum { WO_ENGINE_DEFAULT = 0, WO_ENGINE_SMEM = 1, WO_ENGINE_HYBRID = 2 };
 wo_status wo_schedule_set(int pass, int n, int engine);

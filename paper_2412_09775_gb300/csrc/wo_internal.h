@@ -225,8 +225,8 @@ int cols_engine(int n);  // WO_ENGINE_SMEM or WO_ENGINE_HYBRID
 // The x and y transforms of a plane in one kernel per direction (wo_xy.cu),
 // and the helpers that pick it or the two passes by the schedule table.
 bool xy_supported(int X, int Y);
-int xy_engine(int X, int Y);
-int xy_engine_for(int X, int Y, long long planes);  // WO_ENGINE_HYBRID: the fused kernels
+int xy_engine(int X, int Y);                        // WO_ENGINE_HYBRID: the fused kernels
+int xy_engine_for(int X, int Y, long long planes);  // an operator's pass over that many planes
 cudaError_t xy_fwd(int X, int Y, const float* in, float2* out, long long nplanes, RowBg bg, cudaStream_t s);
 cudaError_t xy_inv(int X, int Y, const float2* in, float* out, long long nplanes, float scale, RowBg bg,
                    cudaStream_t s);

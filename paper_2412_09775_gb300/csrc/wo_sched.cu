@@ -28,32 +28,28 @@ std::atomic<int> g_xy_engine[kMaxLen + 1];     // 0: default, keyed by Y (X == Y
 constexpr long long kXyFewPlanes = 768;
 }  // namespace
 
-int xy_engine(int X, int Y) {
-  if (!xy_supported(X, Y)) return WO_ENGINE_SMEM;
-  const int e = g_xy_engine[Y].load(std::memory_order_relaxed);
-  if (e == WO_ENGINE_SMEM || e == WO_ENGINE_HYBRID) return e;
-  // default: the separate x and y passes.  The fused kernels hold a 109 KB
-  // plane tile per CTA, so an SM runs two CTAs of four warps and overlaps
-  // little of one CTA's copies with the other's transforms: 11.87 against
-  // 10.99 ms per step of the 256-tile field (k_xy_fwd 410 us and k_xy_inv
-  // 614 us per 64 tiles under ncu, 8 warps per SM); the autotuner keeps
-  // them where they measure faster
-  return WO_ENGINE_SMEM;
-}
-
-// The engine of an operator's xy passes over `planes` planes.  By default few
-// planes of 64 x 64 take the fused kernels: the launches are what such a call
+// The built-in engine of an operator's xy passes over `planes` planes.  The
+// fused kernels hold a plane tile of up to 109 KB per CTA, so an SM runs two
+// CTAs of four warps and overlaps little of one CTA's copies with the other's
+// transforms: 11.87 against 10.99 ms per step of the 256-tile field (k_xy_fwd
+// 410 us and k_xy_inv 614 us per 64 tiles under ncu, 8 warps per SM).  Few planes
+// of 64 x 64 take them all the same: the launches are what such a call
 // waits for, and two of five fall away (16 to 64 planes 21 -> 17 us a
 // reconstruction, 256 planes 31.9 -> 25.2, 768 planes 47.4 -> 45.6).  Planes of
-// 128 x 128 and 192 x 192 lose even alone (21 -> 30 and 30 -> 47 us: one CTA a
-// plane).
+// 128 x 128 and 192 x 192 lose even alone (21 -> 30 and 30 -> 47 us: two CTAs a
+// plane have too few warps).
+static int xy_builtin(int X, int Y, long long planes) {
+  return X == 64 && Y == 64 && planes <= kXyFewPlanes ? WO_ENGINE_HYBRID : WO_ENGINE_SMEM;
+}
+
 int xy_engine_for(int X, int Y, long long planes) {
   if (!xy_supported(X, Y)) return WO_ENGINE_SMEM;
   const int e = g_xy_engine[Y].load(std::memory_order_relaxed);
-  if (e != WO_ENGINE_SMEM && e != WO_ENGINE_HYBRID && X == 64 && Y == 64 && planes <= kXyFewPlanes)
-    return WO_ENGINE_HYBRID;
-  return xy_engine(X, Y);
+  return e == WO_ENGINE_SMEM || e == WO_ENGINE_HYBRID ? e : xy_builtin(X, Y, planes);
 }
+
+// Without a batch: the engine of many planes.
+int xy_engine(int X, int Y) { return xy_engine_for(X, Y, kXyFewPlanes + 1); }
 
 int recon_engine(int Z, int Y, int X) {
   if (!pipe_supported(Z, Y, X)) return WO_ENGINE_SMEM;
@@ -94,12 +90,14 @@ int rows_engine(int n) {
 // stream s) and keep the faster.  The engines are timed in alternating rounds
 // (kReps runs per round, after one untimed run each) and each keeps its best
 // round, so a clock ramp or a cold cache early on does not decide the
-// choice.  The other engine replaces the built-in default only when it is at
-// least 2 % faster, so near-ties do not flip from one process to the next.
+// choice.  The other engine replaces the built-in one for this batch only when
+// it is at least 2 % faster, so near-ties do not flip from one process to the
+// next; where the built-in one stays, so does the built-in rule (the entry is
+// cleared, and other batches of the length keep what the rule gives them).
 // Returns the engine kept, or -1 on a CUDA error (the entry is then
 // restored).
 template <class Run>
-static int tune_entry(std::atomic<int>& entry, int default_engine, bool hybrid_ok, cudaStream_t s, Run run) {
+static int tune_entry(std::atomic<int>& entry, int builtin, bool hybrid_ok, cudaStream_t s, Run run) {
   constexpr int kEngines = 2, kRounds = 3, kReps = 8;
   const int engines[kEngines] = {WO_ENGINE_SMEM, WO_ENGINE_HYBRID};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -135,10 +133,10 @@ static int tune_entry(std::atomic<int>& entry, int default_engine, bool hybrid_o
   cudaEventDestroy(e1);
   int best = -1;
   for (int k = 0; k < kEngines && !failed; ++k)
-    if (ok[k] && engines[k] == default_engine) best = k;
+    if (ok[k] && engines[k] == builtin) best = k;
   for (int k = 0; k < kEngines && !failed; ++k)
     if (ok[k] && (best < 0 || t_best[k] < 0.98f * t_best[best])) best = k;
-  entry.store(best < 0 ? saved : engines[best]);
+  entry.store(best < 0 ? saved : engines[best] == builtin ? WO_ENGINE_DEFAULT : engines[best]);
   return best < 0 ? -1 : engines[best];
 }
 
@@ -157,7 +155,7 @@ static int tune_xy(int X, long long planes, float2* scratch, cudaStream_t s) {
   float* real = reinterpret_cast<float*>(scratch);
   float2* half = scratch + (size_t)planes * X * X / 2;  // after the real planes
   const RowBg none{};
-  return tune_entry(g_xy_engine[X], WO_ENGINE_SMEM, true, s, [&](int) {
+  return tune_entry(g_xy_engine[X], xy_builtin(X, X, planes), true, s, [&](int) {
     cudaError_t e = plane_xy_fwd(X, X, real, half, planes, none, s);
     if (e != cudaSuccess) return e;
     return plane_xy_inv(X, X, half, real, planes, 1.0f, none, s);
