@@ -66,10 +66,10 @@ CPU_SAMPLE = (96, 256, 256)
 # capture), scaled by 4 to the 256 tiles of a launch of the bench's field
 # (the traffic grows with the tiles).
 NCU_TRAFFIC = {
-    ("field", "tf_arms"): {"bytes": 4 * (34789888 + 458295040), "digest": "a2390ea1d9919fdc"},
-    ("field", "tf_psf_rows"): {"bytes": 4 * (584034048 + 423258624), "digest": "4b80f0aa1abf3e4d"},
-    ("field", "tf_yz"): {"bytes": 4 * (368307712 + 308312576), "digest": "3e5e5d9e0b333553"},
-    ("field", "yz_op"): {"bytes": 4 * (741899264 + 403963136), "digest": "3e5e5d9e0b333553"},
+    ("field", "tf_arms"): {"bytes": 4 * (34908416 + 458464000), "digest": "5e463274f98dff89"},
+    ("field", "tf_psf_rows"): {"bytes": 4 * (584024576 + 423385344), "digest": "826dd987e847cdc2"},
+    ("field", "tf_yz"): {"bytes": 4 * (368271872 + 308166912), "digest": "09fd9f23baa5bd64"},
+    ("field", "yz_op"): {"bytes": 4 * (741788672 + 404317952), "digest": "09fd9f23baa5bd64"},
 }
 
 

@@ -70,8 +70,9 @@ __device__ __forceinline__ int freq_idx(int i, int n) { return (i < (n + 1) / 2)
 // are added together.  Four warps take four rows r of one tile: the geometry
 // of 128 points at a time is formed once for them, and a warp's next plane is
 // its neighbour's plane (L1 hits).  Four points of a lane have their loads in
-// flight at once.  256 x 48x128x128: 1374 -> 472 us (two lanes a slot, half the
-// warps an SM: 616; a slot a lane, the geometry formed by every warp: 945).
+// flight at once.  256 x 48x128x128: 1374 -> 472 us, five CTAs an SM by shared
+// memory (two lanes a slot, three CTAs: 616; a slot a lane, the geometry formed
+// by every warp: 945).
 constexpr int kFeatRows = 4, kFeatPts = 32 * kFeatRows, kFeatSlots = 8;
 
 // I: the type of an offset in a plane (feat_wide).  RPC: rows a CTA, four, or

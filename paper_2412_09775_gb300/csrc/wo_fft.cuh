@@ -42,8 +42,9 @@ __device__ __forceinline__ float2 mul_mi(float2 a) {
 }
 
 // Complex sums of the butterflies as one packed instruction each (add / sub /
-// fma.rn.f32x2: both parts rounded as the scalar instructions round them, so
-// the transforms' values are the scalar code's).  A packed instruction takes
+// fma.rn.f32x2: each part of a sum rounded as the scalar instruction rounds it;
+// where a sum takes a product, dft3's and dft8's constants, it is in one fma,
+// so a transform differs from the scalar forms below by last bits).  A packed instruction takes
 // one issue slot at the arithmetic rate of two scalar ones (measured: 3.85
 // scalar or 1.98 packed warp instructions per clock and SM), and the
 // register-resident transforms are bound by issue: PSF rows of the gradient

@@ -410,7 +410,9 @@ static cudaError_t launch_psf_pair(const TfArgs& a, cudaStream_t s) {
   constexpr int RPC = kPsfThreads / P::T;
   const long long pairs = (a.row_end - a.row_begin + 1) / 2;
   const unsigned grid = (unsigned)((pairs + RPC - 1) / RPC);
-  if (a.kxm) {  // one kind, Y = X, Z 32 or 48 (16 with X = 64) (checked by the caller)
+  // kx-major: aberrated pupils (the others take wo_tfeven.cu); one kind, Y = X,
+  // Z 32 or 48 (16 with X = 64), checked by the caller
+  if (a.kxm) {
     if constexpr (P::N == 64 || P::N == 128 || P::N == 192) {
       if (a.Y != P::N) return cudaErrorInvalidValue;
       auto go = [&](auto zk) {

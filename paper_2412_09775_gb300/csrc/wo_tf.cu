@@ -31,8 +31,9 @@ namespace wo {
 // One block per RY rows of one tile.  The frequency axes are computed once per
 // block (the same IEEE divisions as the float64 reference); the mask
 // predicates are exact float64 products and sums in the reference's order.
-// eta = sqrt(k_m^2 - |nu|^2) takes a float seed and one float64 Newton
-// correction (relative error ~1e-14, far below the float phase resolution).
+// eta = sqrt(k_m^2 - |nu|^2) takes a float seed and its correction from the
+// float64 remainder, kept as an exact float pair (relative error ~1e-14, far
+// below the float phase resolution).
 // Rows per block: between 8 and 32, as many as keep about two blocks per SM
 // busy (each block computes the x frequency axis once, with IEEE divisions).
 constexpr int kRecRowsMax = 32;
