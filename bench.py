@@ -106,6 +106,39 @@ def band_columns(o, X):
     return min(X, 2 * k + 1)
 
 
+EVEN_LENGTHS = (32, 48, 64, 96, 128, 192, 256, 512)  # sides of banks that take the passes of an even pupil
+
+
+def even_arm_bytes(o, kinds, Z, Y, X):
+    """Bytes of one tile's arms as the passes of an even (unaberrated) pupil store
+    and read them: the detection arms' columns k_x >= 0, the source arm's columns
+    that the source reaches (one column of margin; k_x >= 0 on axis), and of an arm
+    that is even in y (fluorescence; all of them on axis) the rows 0 .. Y/2."""
+    k = (band_columns(o, X) - 1) // 2
+    px, lam = X * o["pixel_um"], o["lambda_um"]
+    lo, hi = -k, k
+    if not o.get("smooth_source"):
+        lo = max(lo, int(np.floor((o["tilt_x"] - o["na_ill"]) / lam * px)) - 1)
+        hi = min(hi, int(np.ceil((o["tilt_x"] + o["na_ill"]) / lam * px)) + 1)
+    axial = o["tilt_x"] == 0 and o["tilt_y"] == 0
+    rows, cells = Y // 2 + 1 if axial else Y, 0
+    if {"phase", "absorption"} & set(kinds):
+        cells += rows * (max(hi - (0 if axial else lo) + 1, 0) + k + 1)
+    if "fluor" in kinds:
+        cells += (Y // 2 + 1) * (k + 1)
+    return Z * cells * 8
+
+
+def bank_bytes(o, kinds, Z, Y, X):
+    """The arm and PSF-row passes' bytes of one tile's bank (unaberrated)."""
+    if Y in EVEN_LENGTHS and X in EVEN_LENGTHS:
+        arms = even_arm_bytes(o, kinds, Z, Y, X)
+    else:
+        n_arms = (2 if {"phase", "absorption"} & set(kinds) else 0) + ("fluor" in kinds)
+        arms = n_arms * Z * Y * band_columns(o, X) * 8
+    return {"tf_arms": arms, "tf_psf_rows": arms + len(kinds) * Z * Y * (X // 2 + 1) * 8}
+
+
 def support_columns(o, kinds, Y, X):
     """(k_y, k_x) columns of the half spectrum inside the TFs' support disk,
     (k_y/Y)^2 + (k_x/X)^2 <= r^2 with r = R p + 2/min(Y, X) (cycles per pixel;
@@ -155,7 +188,9 @@ def support_xcols(o, kinds, X):
 
 
 def algorithmic_bytes(shape, kinds, o):
-    """Compulsory HBM bytes per launch of each kernel family for one step."""
+    """Compulsory HBM bytes per launch of each kernel family for one step, the
+    arm and PSF-row passes' as the general ones (any pupil) move them; bank_bytes
+    has an unaberrated bank's."""
     Z, Y, X = shape
     Xh = X // 2 + 1
     nk = len(kinds)
@@ -641,7 +676,7 @@ def report(args, world, ms_max, e2e_ms, prof, launches, clk, tune=None, lib=None
     vox = float(Z * Y * X)
     value = job_throughput(vox, world, ms_max)
     import phantom as ph
-    algo = algorithmic_bytes(SHAPE, KINDS, ph.optics())
+    algo = dict(algorithmic_bytes(SHAPE, KINDS, ph.optics()), **bank_bytes(ph.optics(), KINDS, *SHAPE))
     per_kernel = {}
     for name, (cnt, tot) in prof.items():
         avg = tot / cnt if cnt else 0.0
@@ -741,12 +776,11 @@ def field_algorithmic_bytes(o_list, Z, E, field_vox):
     out = {k: 0 for k in ("tf_pupil_record", "tf_arms", "tf_psf_rows", "tf_ypass", "tf_zpass", "tf_yz", "rows_r2c",
                           "y_fwd", "xy_fwd", "z_fused", "yz_op", "y_inv", "rows_c2r", "xy_inv")}
     for o in o_list:
-        arms = 2 * Z * E * band_columns(o, E) * 8
+        for name, b in bank_bytes(o, ("phase",), Z, E, E).items():
+            out[name] += b
         inside = Z * support_columns(o, ("phase",), E, E) * 8
         planes_in = support_planes(o, ("phase",), E)
         out["tf_pupil_record"] += E * E * 16
-        out["tf_arms"] += arms
-        out["tf_psf_rows"] += arms + half
         out["tf_ypass"] += 2 * half
         out["tf_zpass"] += 2 * half
         out["tf_yz"] += 2 * planes_in * Z * E * 8  # the plane engine: the TF planes inside the support in and out
@@ -1247,11 +1281,13 @@ TUNE_WORKLOAD = {
 def tune_algorithmic_bytes(o, n, n_params):
     """Compulsory HBM bytes per launch of each kernel family of one Adam step
     over n tiles: 4 arms and 2 per-plane TF slots for the defocus alone, 7
-    arms and 5 slots for the four parameters (no z transform)."""
+    arms and 5 slots for the four parameters (no z transform); two of the arms,
+    B and B', are even in k_x and have their columns k_x >= 0 alone."""
     Z, Y, X = TUNE_SHAPE
     half = Z * Y * (X // 2 + 1) * 8
     n_arms, n_slots = (4, 2) if n_params == 1 else (7, 5)
-    arms = n_arms * Z * Y * band_columns(o, X) * 8
+    band = band_columns(o, X)
+    arms = Z * Y * ((n_arms - 2) * band + 2 * ((band - 1) // 2 + 1)) * 8
     return {k: n * v for k, v in {
         "tf_pupil_record": Y * X * (16 if n_params == 1 else 32), "tf_arms": arms,
         "tf_psf_rows": arms + n_slots * half, "tf_ypass": 2 * n_slots * half,
