@@ -527,6 +527,14 @@ def profiled_pass(B, step, n):
     return B.wo_profile_read()
 
 
+def step_profile(B, step, warmup=3, n=5):
+    """Per-kernel launches and milliseconds of one step: n profiled ones after
+    `warmup` that are not (the first pays for loading its kernels)."""
+    for _ in range(warmup):
+        step()
+    return {k: (c // n, t / n) for k, (c, t) in profiled_pass(B, step, n).items()}
+
+
 def run_e2e(args, B, o, data, out, tf, ws, stream, barrier, world, dev):
     """Steps through the public API from pinned host buffers: each step copies
     its two input stacks to the device, builds the TFs, reconstructs and
@@ -1383,13 +1391,8 @@ def autotune_leg(args, rank, world, local_rank, with_cpu=True):
         B.wo_autotune(n, Z, Y, X, pb.kinds, pb.ws)  # the workspace is scratch between calls
     sched = A.default_schedule4(truth[0]) if four else A.default_schedule(truth[0])
     n_adam = sum(p.steps for p in sched)
-    # per-kernel times of one eager Adam step on the full loss
-    B.wo_profile_read()
-    B.wo_profile_enable(True)
-    pb.step(0.0, 0.0)
-    torch.cuda.synchronize()
-    B.wo_profile_enable(False)
-    prof = B.wo_profile_read()
+    # per-kernel times of an eager Adam step on the full loss
+    prof = step_profile(B, lambda: pb.step(0.0, 0.0))
     per_adam_step = sum(c for c, _ in prof.values())  # library launches of one Adam step
     pb.run(sched, graph=True)  # captures (and replays once)
     per_run = n_adam * per_adam_step
