@@ -66,10 +66,10 @@ CPU_SAMPLE = (96, 256, 256)
 # capture), scaled by 4 to the 256 tiles of a launch of the bench's field
 # (the traffic grows with the tiles).
 NCU_TRAFFIC = {
-    ("field", "tf_arms"): {"bytes": 4 * (34908416 + 458464000), "digest": "5e463274f98dff89"},
-    ("field", "tf_psf_rows"): {"bytes": 4 * (584024576 + 423385344), "digest": "826dd987e847cdc2"},
-    ("field", "tf_yz"): {"bytes": 4 * (368271872 + 308166912), "digest": "09fd9f23baa5bd64"},
-    ("field", "yz_op"): {"bytes": 4 * (741788672 + 404317952), "digest": "09fd9f23baa5bd64"},
+    ("field", "tf_arms"): {"bytes": 4 * (34795520 + 458251776), "digest": "5e463274f98dff89"},
+    ("field", "tf_psf_rows"): {"bytes": 4 * (584092672 + 423304704), "digest": "826dd987e847cdc2"},
+    ("field", "tf_yz"): {"bytes": 4 * (368269568 + 308192512), "digest": "3ebe8577580a6a98"},
+    ("field", "yz_op"): {"bytes": 4 * (741488384 + 404006912), "digest": "3ebe8577580a6a98"},
 }
 
 

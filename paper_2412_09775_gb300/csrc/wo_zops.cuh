@@ -2,8 +2,8 @@
 // inverse z transform, in one kernel (shared by the translation units that
 // instantiate it).
 //
-// Up to 192 planes the stages run through registers (k_z_thru below; z_thru()
-// says where); the other lengths take the shared-memory form (k_z_fused),
+// Up to 192 planes the stages run through registers (k_z_thru below;
+// launch_z_fused says where); the other lengths take the shared-memory form (k_z_fused),
 // described here.  A CTA owns B adjacent x columns of one (tile, y) row of the
 // half-spectrum volumes.  The z columns of all NI input volumes are copied
 // asynchronously into shared memory laid out [n][slot][b], so one batched
@@ -515,22 +515,28 @@ __global__ void __launch_bounds__(ZGeom<N, NI>::NT, ZGeom<N, NI>::MINB)
 // shared memory: the first stage, three butterflies a column, then leaves up to
 // five threads in eight of a CTA without a load (24 planes, 61 x 128x128: 65 us,
 // through registers 88; 15 x 256x256: 59, 82; 12 planes of 256x256: 56, 62).
-// With two or three volumes every thread loads.
+// With two or three volumes every thread loads; and a bank of more slots than
+// the one in use (a derivative bank) would be copied whole (2 x 24x256x256: 48.5
+// us a reconstruction, through registers 46.9).
 template <int N, int NI, int NO>
-constexpr bool z_thru() {
-  return N > 1 && N <= 192 && !(NI == 1 && NO == 1 && (N == 12 || N == 24));
+constexpr bool z_idle() {
+  return NI == 1 && NO == 1 && (N == 12 || N == 24);
 }
 
 template <int N, int NI, int NO>
 cudaError_t launch_z_fused(const float2* in, float2* out, const float2* tf, ZOp op, int n_tiles, int Y, int Xh,
                            cudaStream_t s) {
-  if constexpr (z_thru<N, NI, NO>()) {
-    using G = ZThruGeom<N, NI, NO>;
-    const cudaError_t attr = allow_smem(k_z_thru<N, NI, NO>, G::SMEM);
-    if (attr != cudaSuccess) return attr;
-    dim3 grid((unsigned)((Y * Xh + G::B - 1) / G::B), (unsigned)n_tiles);
-    WO_LAUNCH("z_fused", s, (k_z_thru<N, NI, NO><<<grid, G::NT, G::SMEM, s>>>(in, out, tf, op, Y, Xh)));
-  } else {
+  if constexpr (N > 1 && N <= 192) {
+    if (!z_idle<N, NI, NO>() || op.n_tf > 1) {
+      using G = ZThruGeom<N, NI, NO>;
+      const cudaError_t attr = allow_smem(k_z_thru<N, NI, NO>, G::SMEM);
+      if (attr != cudaSuccess) return attr;
+      dim3 grid((unsigned)((Y * Xh + G::B - 1) / G::B), (unsigned)n_tiles);
+      WO_LAUNCH("z_fused", s, (k_z_thru<N, NI, NO><<<grid, G::NT, G::SMEM, s>>>(in, out, tf, op, Y, Xh)));
+      return cudaGetLastError();
+    }
+  }
+  if constexpr (N <= 1 || N > 192 || z_idle<N, NI, NO>()) {
     using G = ZGeom<N, (NI > NO ? NI : NO)>;
     const cudaError_t attr = allow_smem(k_z_fused<N, NI, NO>, G::SMEM_TF);
     if (attr != cudaSuccess) return attr;
