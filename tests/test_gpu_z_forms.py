@@ -42,14 +42,15 @@ def bank(env, kinds, n, Z, E, **kw):
     return ol, tf, ws
 
 
-@pytest.mark.parametrize("n,E", [(61, 128), (15, 256)])
-def test_one_volume_of_24_planes(env, n, E):
-    """1.35 to 1.6 row passes in shared memory, 1.9 to 2.1 through registers."""
+@pytest.mark.parametrize("n,E,limit", [(61, 128, 1.95), (15, 256, 1.63)])
+def test_one_volume_of_24_planes(env, n, E, limit):
+    """1.66 and 1.38 row passes in shared memory, 2.24 and 1.89 through registers:
+    the limits lie halfway."""
     B, torch, dev = env
     _, tf, ws = bank(env, 1, n, 24, E)
     d, out = torch.randn((n, 1, 24, E, E), device=dev), torch.empty((n, 1, 24, E, E), device=dev)
     t = times(env, lambda: B.wo_reconstruct(tf, 1, d, None, [1e-3], B.WO_ETA_RELATIVE, B.WO_MODE_3D, out, n, 24, E, E, ws))
-    assert t["z_fused"] <= 1.75 * t["rows_r2c"], t
+    assert t["z_fused"] <= limit * t["rows_r2c"], t
 
 
 @pytest.mark.parametrize("kinds,n,Z,E", [(7, 1, 96, 512), (3, 12, 24, 256), (5, 19, 16, 256)])
